@@ -131,6 +131,19 @@ __device__ __forceinline__ void tc_mma_ta(uint32_t d_tmem, uint32_t a_tmem, uint
         : "memory");
 }
 
+// One lane of the (converged) warp.  The MMAs are issued under this predicate, not under
+// `lane == 0`: the compiler then knows that a single thread issues and keeps the descriptors in
+// uniform registers.  Measured alone (M = 128, K = 16, 128-byte rows): an instruction takes N / 2
+// cycles (N = 112: 62, 224: 114) either way, but with 25 other warps storing to shared memory
+// 138 cycles whatever its N under `lane == 0`, and unchanged under elect.  N = 84, F = 4,
+// E = 2^20, three terms: 951 -> 791 us; N = 120, F = 3, E = 310977: 439 -> 345 us.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.b32 %0, 1, 0, p;\n}\n" : "=r"(r));
+    return r != 0;
+}
+
 // Shared-memory matrix descriptor, K-major, swizzle atom of W bytes per row (32, 64, 128):
 // start address, leading offset 16 B (unused for swizzled K-major), stride between
 // 8-row groups = 8*W, descriptor version 1, layout type per swizzle width.
@@ -435,7 +448,10 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
             const uint64_t ad = a0 + ((uint32_t)(at * termA + kb * TE * W) >> 4);
             const uint64_t bd = b0 + ((uint32_t)(brow * W + kb * bkb) >> 4);
             const uint32_t at_tm = a_tmb + (uint32_t)(at * (Kn / 2) + kb * KB / 2);
-            for (int ki = 0; ki < steps; ++ki) {
+#pragma unroll
+            for (int ki = 0; ki < 4; ++ki) {  // at most four K steps of 16 in a K-block of 64
+                if (ki >= steps)
+                    break;
                 if (kATmem && a.a_tmem)
                     tc_mma_ta(dtm + dcol, at_tm + 8u * ki, bd + 2 * ki, id, accumulate);
                 else
@@ -462,7 +478,7 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
                             break;
                         tc_fence_after();
                     }
-                    if (lane == 0) {
+                    if (elect_one()) {
                         const uint32_t acc = kb > 0;  // block 0 of a region's first product overwrites
                         if (NT == 1) {
                             mma_block(dtm, a0, b0, kb, 0, 0, idesc, 0, acc);
@@ -493,7 +509,7 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
                     fail();
                 break;
             }
-            if (lane == 0)
+            if (elect_one())
                 tc_commit(&acc_full[b]);
             __syncwarp();
             if (*abort_flag)
