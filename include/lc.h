@@ -110,7 +110,7 @@ struct lc_variant {
     uint32_t struct_size;     /* sizeof(lc_variant) */
     int32_t engine;           /* LC_ENGINE_*: SIMT FMA tiles, tcgen05 tensor cores, one warp
                                  per element group with shuffles (small N), or K-split SIMT
-                                 (FP32): 8 x 8 register blocks over a tile_e x 128 output
+                                 (FP32): 8 x 8 register blocks over a tile_e x (64 to 128) output
                                  block, the j reduction cut into chunks of `unroll` (8 or 16)
                                  whose D^T rows are fetched one chunk ahead, so D^T need not
                                  fit in shared memory; tile_e 64 or 128, elems_per_thread =
@@ -168,7 +168,7 @@ struct lc_variant {
 /*
  * A reasonable descriptor for (E, N, F, layout, precision): fills *v.  The choices follow
  * the autotuner's measurements on this GPU: FP32 on the warp engine up to N = 12, SIMT
- * tiles below N = 96, the K-split engine from N = 96; BF16 and BF16X3 on the tensor cores
+ * tiles below N = 64, the K-split engine from N = 64; BF16 and BF16X3 on the tensor cores
  * (BF16X3 with the A terms in shared memory, from about N = 100 to 128 in tensor memory),
  * and where no tensor-core plan exists the FP32 kernels, whose error is below both
  * reduced-precision bounds; FP64 SIMT tiles.  No GPU work is done.
@@ -425,7 +425,7 @@ lc_status lc_grouped_workspace_size(const lc_kernel *k, const lc_variant *v, con
  * column block) unit gets at least one CTA, and the rest go to the unit whose estimated
  * time (tiles x per-tile cost / CTAs) is the largest.  More units than SMs is
  * LC_ERR_INVALID_VARIANT.  Groups without a tensor-core plan (e.g. N above the plans'
- * limit) run after it, each in a K-split FP32 launch (tiles of 128 elements, j chunks of 8,
+ * limit) run after it, each in a K-split FP32 launch (tiles of 128 elements, j chunks of 16,
  * one u buffer), or, without a K-split plan, in a FP32 SIMT grouped launch (8 x 8 register
  * blocks, unroll 4, two stages, three CTAs per SM); their results are FP32's, below both
  * reduced-precision bounds.

@@ -1314,18 +1314,19 @@ static lc_status resolve(const Kernel &K, long long E, int N, int F, const lc_va
         k.C = F * N;
         k.Kp = (N + BK - 1) / BK * BK;
         k.nkc = k.Kp / BK;
-        k.nblocks = (k.C + 127) / 128;
+        k.bn = ks_block_cols(k.C, BM);
+        k.nblocks = (k.C + k.bn - 1) / k.bn;
         k.ntiles = (E + BM - 1) / BM;
         k.ubufs = v->stages;
         k.vec_u = node && E % 4 == 0;
         k.vec_out = node ? E % 4 == 0 : N % 4 == 0;
         r.ks_bm = BM;
         r.ks_bk = BK;
-        const size_t smem = ks_smem_bytes(k.Kp, BM, BK, k.ubufs);
+        const size_t smem = ks_smem_bytes(k.Kp, BM, BK, k.bn, k.ubufs);
         if (smem > smem_cap)
             return LC_ERR_INVALID_VARIANT;
         // resident CTAs per SM: the descriptor's, else as many as shared memory allows (at
-        // most 2 of 256 threads or 3 of 128: the register bound of the instances)
+        // most 2 of 128 or 3 of 64 elements: the register bound of the instances)
         int cps = (int)std::min<size_t>((smem_cap + 1024) / (smem + 1024), BM == 128 ? 2 : 3);
         if (v->ctas_per_sm > 0)
             cps = std::min(cps, v->ctas_per_sm);
@@ -1335,7 +1336,7 @@ static lc_status resolve(const Kernel &K, long long E, int N, int F, const lc_va
             return LC_ERR_INVALID_VARIANT;
         SimtGeom &g = r.g;
         g.grid = (int)grid;
-        g.threads = BM / 8 * 16;
+        g.threads = ks_threads(BM, k.bn);
         g.smem = smem;
         g.TE = BM;
         g.ntiles = k.ntiles;
@@ -1829,16 +1830,19 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
         d.tile_e = 64;
         d.stages = 2;
     } else if (precision == LC_PREC_FP32) {
-        if (precision == LC_PREC_FP32 && N >= 96) {
-            // large N: the K-split kernel (D^T streamed in chunks) measured faster than the
-            // SIMT kernel holding all of D^T (N = 120: 0.69 against 0.86 ms; N = 165: 2.6
-            // against 3.6 ms)
+        if (N >= 64) {
+            // large N: the K-split kernel (D^T streamed in chunks of 16 j) against the SIMT
+            // kernel holding all of D^T: N = 64, F = 3, E = 2^19 392 against 476 us element-major,
+            // 318 against 345 node-major; N = 84, F = 4, E = 2^20 1565 against 1746 and 1342
+            // against 2125; at N = 56 they are within 5 % of one another.  Tiles of 128 elements,
+            // or of 64 where those would not give every SM a CTA (N = 120, F = 3, E = 9000: 35
+            // against 48 us).
             lc_variant k = d;
             k.engine = LC_ENGINE_KSPLIT;
-            k.tile_e = 128;
+            k.tile_e = (E + 127) / 128 < 152 ? 64 : 128;
             k.elems_per_thread = 8;
             k.split_i = 8;
-            k.unroll = 8;
+            k.unroll = 16;
             k.prefetch_smem = 1;
             k.stages = 1;
             if (lc_variant_validate(kh, E, N, F, &k) == LC_OK) {
@@ -2672,7 +2676,7 @@ struct GroupedPlanAll {
 
 // The K-split descriptor for the groups of a grouped plan that run as their own K-split
 // launch: tensor-core plans' groups without any tensor-core plan (N above 128 for three
-// terms), FP32 plans' groups of N >= 96 (tiles of 128 elements, j chunks of 8, one u buffer:
+// terms), FP32 plans' groups of N >= 96 (tiles of 128 elements, j chunks of 16, one u buffer:
 // the fastest measured for N = 120 and 165).
 static lc_variant grouped_ks_fallback(const lc_variant *v)
 {
@@ -2685,7 +2689,7 @@ static lc_variant grouped_ks_fallback(const lc_variant *v)
     s.tile_e = 128;
     s.elems_per_thread = 8;
     s.split_i = 8;
-    s.unroll = 8;
+    s.unroll = 16;
     s.prefetch_smem = 1;
     s.stages = 1;
     return s;

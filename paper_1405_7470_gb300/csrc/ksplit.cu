@@ -12,19 +12,37 @@
 //   add_prefetch(u)          the u tile, transposed to [j][e], stays resident for every
 //                            column block of the tile; with two buffers the next tile's
 //                            u is fetched while this one is used.
-//   ilp on e and on i        8 x 8 register block per thread: elements {4ty..4ty+3,
-//                            BM/2+4ty..}, columns {4tx..4tx+3, 64+4tx..} of a 128-column
-//                            block; the operand reads are 16-byte vector loads.
+//   ilp on e and on i        8 x 8 register block per thread: two quads of tile positions by
+//                            two quads of column positions; the operand reads are 16-byte
+//                            vector loads.
 //   unr on j                 the chunk loop is fully unrolled.
-// Column blocks of 128 cover F*N columns; the u tile is read once per tile for all of them.
+// Column blocks of BN (64 to 128) cover the F*N columns; the u tile is read once per tile
+// for all of them.
+//
+// What bounds it: the FMA pipes (70 % busy at N = 120; the 8 x 8 outer product alone, from
+// shared memory, reaches 63 TFLOP/s of the 80.5 derived).  The rest must stay out of its way:
+//   multiply-adds packed in pairs along the columns (f32x2): the pipes take as long, but half
+//                 the issue slots are left for everything else.  Without the next point
+//                 they gained nothing.
+//   D^T chunks    neighbouring lanes read neighbouring j of one D row (BK lanes per row, 32 /
+//                 BK rows per request).  One column per two lanes, as this kernel had it,
+//                 touched 16 rows per request and kept the load/store pipe busy for about as
+//                 long as the FMAs themselves.
+//   chunk length  16 j (one barrier per 16) beats 8: N = 120, node-major, 617 against 668 us.
+//   stores        neighbouring threads hold neighbouring values of the output's contiguous
+//                 axis.  Where 16-byte stores are aligned each thread's quads are four
+//                 consecutive values; otherwise the positions are permuted so that a quad is
+//                 every T-th value (T threads along that axis) and each 4-byte store of a
+//                 warp writes runs of T consecutive values.
+// Measured before -> after: N = 120, F = 3, E = 310977 node-major 889 -> 603 us; N = 165, F = 3,
+// E = 564445 element-major 2584 -> 2114 us; N = 84, F = 4, E = 2^20 element-major 1790 -> 1565 us,
+// node-major 1342 us (45 to 50 TFLOP/s with the padding counted).
 #include <cuda_runtime.h>
 
 #include "lc_internal.h"
 #include "tma.cuh"
 
 namespace lc {
-
-static constexpr int kKsBN = 128;  // output columns per block
 
 // 4-byte asynchronous copy global -> shared; `bytes` 0 writes a zero (nothing is read).
 __device__ __forceinline__ void cp_async4(float *dst, const float *src, uint32_t bytes)
@@ -43,20 +61,43 @@ __device__ __forceinline__ void cp_async16(float *dst, const float *src, uint32_
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-template <int LAYOUT, int BM, int BK>
+template <int BM, int BK, int BN>
 struct KsShape {
-    static constexpr int TH = BM / 8 * 16;  // threads: (BM / 8) x 16
-    static constexpr int LDA = BM + 4;      // u tile row (one j): BM elements, padded
-    static constexpr int LDB = kKsBN + 4;   // D^T chunk row (one j): 128 columns, padded
-    static constexpr int TPC = TH / kKsBN;  // threads per column of a D^T chunk (1 or 2)
-    static constexpr int KPT = BK / TPC;    // chunk rows each of them copies
+    static constexpr int TX = BN / 8;        // threads along the columns
+    static constexpr int TY = BM / 8;        // threads along the elements
+    static constexpr int TH = TX * TY;       // threads of the CTA
+    static constexpr int LDA = BM + 4;       // u tile row (one j): BM positions, padded
+    static constexpr int LDB = BN + 4;       // D^T chunk row (one j): BN positions, padded
+    static constexpr int PP = TH / BK;       // column positions one pass of the CTA's threads copies
+    static constexpr int QB = BN / PP;       // passes over a chunk
+    static_assert(TH % BK == 0 && BN % PP == 0, "a chunk is copied in whole passes");
 };
 
-// Copy the u tile of elements e0 .. e0+BM-1 into ut[j][e] (j < Kp; zeros past N or E).
-template <int LAYOUT, int BM, int BK>
+// The value (0 .. 8T - 1) a position of a tile row holds, for T threads along the row that read
+// the quads 4t .. 4t + 3 of each half.  Permuted: thread t's quad is t, t + T, t + 2T, t + 3T.
+template <int T>
+__device__ __forceinline__ int ks_value(int p, bool perm)
+{
+    if (!perm)
+        return p;
+    const int h = p / (4 * T), q = p - h * 4 * T;
+    return h * 4 * T + q / 4 + (q % 4) * T;
+}
+// The inverse: the position of value v.
+template <int T>
+__device__ __forceinline__ int ks_position(int v, bool perm)
+{
+    if (!perm)
+        return v;
+    const int h = v / (4 * T), q = v - h * 4 * T;
+    return h * 4 * T + (q % T) * 4 + q / T;
+}
+
+// Copy the u tile of elements e0 .. e0+BM-1 into ut[j][position of e] (j < Kp; zeros past N or E).
+template <int LAYOUT, int BM, int BK, int BN>
 __device__ __forceinline__ void ks_load_u(const KsArgs &a, float *ut, long long e0, int tid)
 {
-    using S = KsShape<LAYOUT, BM, BK>;
+    using S = KsShape<BM, BK, BN>;
     const int N = a.N, Kp = a.Kp;
     const long long E = a.E;
     if (LAYOUT == LC_LAYOUT_NODE_MAJOR) {
@@ -73,7 +114,8 @@ __device__ __forceinline__ void ks_load_u(const KsArgs &a, float *ut, long long 
             for (int idx = tid; idx < Kp * BM; idx += S::TH) {
                 const int j = idx / BM, e = idx - j * BM;
                 const bool ok = j < N && e0 + e < E;
-                cp_async4(ut + j * S::LDA + e, ok ? a.u + (size_t)j * E + e0 + e : a.u, ok ? 4u : 0u);
+                cp_async4(ut + j * S::LDA + ks_position<S::TY>(e, !a.vec_out), ok ? a.u + (size_t)j * E + e0 + e : a.u,
+                          ok ? 4u : 0u);
             }
         }
     } else {
@@ -94,69 +136,72 @@ __device__ __forceinline__ void ks_load_u(const KsArgs &a, float *ut, long long 
     }
 }
 
-// Copy rows kc*BK .. kc*BK+BK-1 of the D^T column block starting at column c0 into bs[k][c].
-// Each thread copies KPT rows of one column: `drow` is that column's D row (null past C).
-template <int LAYOUT, int BM, int BK>
-__device__ __forceinline__ void ks_load_b(const KsArgs &a, float *bs, const float *drow, int kc, int tid)
-{
-    using S = KsShape<LAYOUT, BM, BK>;
-    const int cl = tid / S::TPC, k0 = (tid - cl * S::TPC) * S::KPT;
+// The D^T chunks of one column block.  D read as [F*N][N] has one row per column of D^T.  Lane ->
+// (k = tid % BK, position tid / BK + PP q): BK consecutive j of a row per 32 / BK positions.  What
+// depends on the column block only is kept from chunk to chunk: per copy an add and a select
+// remain (computing the columns in every chunk cost 20 integer instructions a copy).
+template <int BM, int BK, int BN>
+struct KsB {
+    using S = KsShape<BM, BK, BN>;
+    int off[S::QB];  // the copy's D offset in the block's first chunk (0 past the last column)
+    uint32_t valid;  // bit q: the copy's column exists
+
+    __device__ __forceinline__ void block(const KsArgs &a, int cb, int tid, bool perm)
+    {
+        const int k = min(tid % BK, a.N - 1), p0 = tid / BK;
+        valid = 0;
 #pragma unroll
-    for (int q = 0; q < S::KPT; ++q) {
-        const int j = kc * BK + k0 + q;
-        const bool ok = drow != nullptr && j < a.N;
-        cp_async4(bs + (k0 + q) * S::LDB + cl, ok ? drow + j : a.D, ok ? 4u : 0u);
+        for (int q = 0; q < S::QB; ++q) {
+            const int c = cb * BN + ks_value<S::TX>(p0 + S::PP * q, perm);
+            off[q] = c < a.C ? c * a.N + k : 0;
+            valid |= (c < a.C ? 1u : 0u) << q;
+        }
     }
-}
+    // rows kc*BK .. kc*BK+BK-1 into bs[k][position], zeros past N or past the last column
+    __device__ __forceinline__ void load(const KsArgs &a, float *bs, int kc, int tid) const
+    {
+        const int k = tid % BK;
+        const bool in = kc * BK + k < a.N;
+        const uint32_t ok = in ? valid : 0u;
+        const float *src = a.D + (in ? kc * BK : 0);
+        float *dst = bs + k * S::LDB + tid / BK;
+#pragma unroll
+        for (int q = 0; q < S::QB; ++q)
+            cp_async4(dst + S::PP * q, src + off[q], (ok >> q & 1u) * 4u);
+    }
+};
 
-// The D row feeding column cl of block cb (null past the last column): column c = f*N + i
-// reads D[f][i][:].
-__device__ __forceinline__ const float *ks_drow(const KsArgs &a, int cb, int cl)
-{
-    const int c = cb * kKsBN + cl;
-    if (c >= a.C)
-        return nullptr;
-    const int f = c / a.N, i = c - f * a.N;
-    return a.D + ((size_t)f * a.N + i) * a.N;
-}
-
-// Resident CTAs the register budget is sized for (128 registers a thread at 2 x 256 or
-// 3 x 128 threads).
-#ifndef KS_MIN_CTAS_128
-#define KS_MIN_CTAS_128 2
-#endif
-#ifndef KS_MIN_CTAS_64
-#define KS_MIN_CTAS_64 3
-#endif
-
-template <int LAYOUT, int BM, int BK>
-__global__ void __launch_bounds__(BM / 8 * 16, BM == 128 ? KS_MIN_CTAS_128 : KS_MIN_CTAS_64)
+template <int LAYOUT, int BM, int BK, int BN>
+__global__ void __launch_bounds__(KsShape<BM, BK, BN>::TH, BM == 128 ? 2 : 3)
     ks_contract_kernel(const __grid_constant__ KsArgs a)
 {
-    using S = KsShape<LAYOUT, BM, BK>;
+    using S = KsShape<BM, BK, BN>;
     constexpr bool NODE = LAYOUT == LC_LAYOUT_NODE_MAJOR;
     extern __shared__ __align__(16) float ks_smem[];
     const int N = a.N, Kp = a.Kp, nkc = a.nkc, nb = a.nblocks;
     const long long E = a.E;
     float *ubuf = ks_smem;                                    // [ubufs][Kp][LDA]
     float *bbuf = ks_smem + (size_t)a.ubufs * Kp * S::LDA;    // [2][BK][LDB]
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    const int cl = tid / S::TPC;  // the D^T column this thread copies
+    // the threads of a warp run along the output's contiguous axis
+    const int tid = threadIdx.x;
+    const int tx = NODE ? tid / S::TY : tid % S::TX, ty = NODE ? tid % S::TY : tid / S::TX;
+    const bool permc = !NODE && !a.vec_out;  // column positions permuted (element-major, N % 4 != 0)
     const long long t0 = blockIdx.x, dt = gridDim.x;
     if (t0 >= a.ntiles)
         return;
 
-    float acc[8][8];
+    uint64_t acc2[8][4];  // acc2[x][p]: columns 2p and 2p + 1 of the thread's eight, packed
 #pragma unroll
     for (int x = 0; x < 8; ++x)
 #pragma unroll
-        for (int y = 0; y < 8; ++y)
-            acc[x][y] = 0.f;
+        for (int p = 0; p < 4; ++p)
+            acc2[x][p] = 0;
 
     // prologue: the first tile's u and the first chunk
-    const float *drow = ks_drow(a, 0, cl);
-    ks_load_u<LAYOUT, BM, BK>(a, ubuf, t0 * BM, tid);
-    ks_load_b<LAYOUT, BM, BK>(a, bbuf, drow, 0, tid);
+    ks_load_u<LAYOUT, BM, BK, BN>(a, ubuf, t0 * BM, tid);
+    KsB<BM, BK, BN> bsrc;
+    bsrc.block(a, 0, tid, permc);
+    bsrc.load(a, bbuf, 0, tid);
     cp_async_commit();
     int sl = 0;  // ring slot of the current chunk
     int ti = 0;
@@ -171,7 +216,7 @@ __global__ void __launch_bounds__(BM / 8 * 16, BM == 128 ? KS_MIN_CTAS_128 : KS_
                 __syncthreads();      // everyone's landed; everyone is done with the other slot
                 if (a.ubufs == 1 && ti > 0 && cb == 0 && kc == 0) {
                     // one u buffer: the previous tile's reads are over only now
-                    ks_load_u<LAYOUT, BM, BK>(a, ubuf, e0, tid);
+                    ks_load_u<LAYOUT, BM, BK, BN>(a, ubuf, e0, tid);
                     cp_async_commit();
                     cp_async_wait_all();
                     __syncthreads();
@@ -182,126 +227,165 @@ __global__ void __launch_bounds__(BM / 8 * 16, BM == 128 ? KS_MIN_CTAS_128 : KS_
                     nkc_ = 0;
                     ncb = cb + 1;
                 }
-                const bool next_in_tile = ncb < nb;
-                if (next_in_tile || has_next_tile) {
-                    if (ncb == nb)
-                        ncb = 0;
-                    if (nkc_ == 0)
-                        drow = ks_drow(a, ncb, cl);
-                    ks_load_b<LAYOUT, BM, BK>(a, bbuf + (size_t)(sl ^ 1) * BK * S::LDB, drow, nkc_, tid);
+                if (ncb < nb || has_next_tile) {
+                    if (nkc_ == 0 && nb > 1)
+                        bsrc.block(a, ncb == nb ? 0 : ncb, tid, permc);
+                    bsrc.load(a, bbuf + (size_t)(sl ^ 1) * BK * S::LDB, nkc_, tid);
                 }
                 if (a.ubufs == 2 && cb == 0 && kc == 0 && has_next_tile)
-                    ks_load_u<LAYOUT, BM, BK>(a, ubuf + (size_t)(ub ^ 1) * Kp * S::LDA, (t + dt) * BM, tid);
+                    ks_load_u<LAYOUT, BM, BK, BN>(a, ubuf + (size_t)(ub ^ 1) * Kp * S::LDA, (t + dt) * BM, tid);
                 cp_async_commit();
 
-                const float *A = ut + (size_t)kc * BK * S::LDA;
-                const float *B = bbuf + (size_t)sl * BK * S::LDB;
+                const float *A = ut + (size_t)kc * BK * S::LDA + 4 * ty;
+                const float *B = bbuf + (size_t)sl * BK * S::LDB + 4 * tx;
 #pragma unroll
                 for (int k = 0; k < BK; ++k) {
-                    const float4 a0 = *reinterpret_cast<const float4 *>(A + k * S::LDA + 4 * ty);
-                    const float4 a1 = *reinterpret_cast<const float4 *>(A + k * S::LDA + BM / 2 + 4 * ty);
-                    const float4 b0 = *reinterpret_cast<const float4 *>(B + k * S::LDB + 4 * tx);
-                    const float4 b1 = *reinterpret_cast<const float4 *>(B + k * S::LDB + 64 + 4 * tx);
+                    if (BK == 16 && k == 8 && kc * BK + 8 >= N)
+                        break;  // the last chunk's second half holds no node
+                    const float4 a0 = *reinterpret_cast<const float4 *>(A + k * S::LDA);
+                    const float4 a1 = *reinterpret_cast<const float4 *>(A + k * S::LDA + BM / 2);
+                    const ulonglong2 b0 = *reinterpret_cast<const ulonglong2 *>(B + k * S::LDB);
+                    const ulonglong2 b1 = *reinterpret_cast<const ulonglong2 *>(B + k * S::LDB + BN / 2);
                     const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-                    const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+                    const uint64_t bv[4] = {b0.x, b0.y, b1.x, b1.y};
 #pragma unroll
-                    for (int x = 0; x < 8; ++x)
+                    for (int x = 0; x < 8; ++x) {
+                        const uint64_t ax = pack_f32x2(av[x], av[x]);
 #pragma unroll
-                        for (int y = 0; y < 8; ++y)
-                            acc[x][y] = fmaf(av[x], bv[y], acc[x][y]);
+                        for (int p = 0; p < 4; ++p)
+                            acc2[x][p] = fma_f32x2(ax, bv[p], acc2[x][p]);
+                    }
                 }
                 sl ^= 1;
             }
-            // the 8 x 8 block of column block cb: rows 4ty + (0..3) and BM/2 + 4ty + (0..3),
-            // columns 4tx + (0..3) and 64 + 4tx + (0..3)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int c4 = cb * kKsBN + 64 * h + 4 * tx;  // first of 4 consecutive columns
-                if (c4 >= a.C)
-                    continue;
-                if (NODE) {
-                    // out[f][i][e]: per column, 4 consecutive elements
-#pragma unroll
-                    for (int y = 0; y < 4; ++y) {
-                        const int c = c4 + y;
-                        if (c >= a.C)
-                            break;
-                        const int f = c / N, i = c - f * N;
-                        float *col = a.out + ((size_t)f * N + i) * E;
-#pragma unroll
-                        for (int g = 0; g < 2; ++g) {
-                            const long long eb = e0 + g * (BM / 2) + 4 * ty;
-                            const float v0 = acc[4 * g][4 * h + y], v1 = acc[4 * g + 1][4 * h + y];
-                            const float v2 = acc[4 * g + 2][4 * h + y], v3 = acc[4 * g + 3][4 * h + y];
-                            if (a.vec_out && eb + 3 < E) {
-                                *reinterpret_cast<float4 *>(col + eb) = make_float4(v0, v1, v2, v3);
-                            } else {
-                                const float vv[4] = {v0, v1, v2, v3};
-#pragma unroll
-                                for (int z = 0; z < 4; ++z)
-                                    if (eb + z < E)
-                                        col[eb + z] = vv[z];
-                            }
-                        }
-                    }
-                } else {
-                    // out[f][e][i]: per element, 4 consecutive columns (one operator's when
-                    // N % 4 == 0: then one 16-byte store)
-                    const int f4 = c4 / N, i4 = c4 - f4 * N;
-#pragma unroll
-                    for (int x = 0; x < 8; ++x) {
-                        const long long e = e0 + (x < 4 ? 4 * ty + x : BM / 2 + 4 * ty + x - 4);
-                        if (e >= E)
-                            continue;
-                        if (a.vec_out) {
-                            *reinterpret_cast<float4 *>(a.out + ((size_t)f4 * E + e) * N + i4) =
-                                make_float4(acc[x][4 * h], acc[x][4 * h + 1], acc[x][4 * h + 2], acc[x][4 * h + 3]);
-                        } else {
-                            int f = f4, i = i4;
-#pragma unroll
-                            for (int y = 0; y < 4; ++y) {
-                                if (c4 + y < a.C)
-                                    a.out[((size_t)f * E + e) * N + i] = acc[x][4 * h + y];
-                                if (++i == N) {
-                                    i = 0;
-                                    ++f;
-                                }
-                            }
-                        }
-                    }
-                }
-            }
+            float acc[8][8];
 #pragma unroll
             for (int x = 0; x < 8; ++x)
 #pragma unroll
-                for (int y = 0; y < 8; ++y)
-                    acc[x][y] = 0.f;
+                for (int p = 0; p < 4; ++p) {
+                    const float2 v = unpack_f32x2(acc2[x][p]);
+                    acc[x][2 * p] = v.x;
+                    acc[x][2 * p + 1] = v.y;
+                    acc2[x][p] = 0;
+                }
+            // store the 8 x 8 block: acc[4g + z][4h + y] is element e0 + g BM/2 + .., column
+            // cb BN + h BN/2 + ..
+            if (NODE) {
+                // out[f][i][e] = column c, contiguous in e
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int y = 0; y < 4; ++y) {
+                        const int c = cb * BN + h * (BN / 2) + 4 * tx + y;
+                        if (c >= a.C)
+                            break;
+                        float *col = a.out + (size_t)c * E;  // (f N + i) E
+#pragma unroll
+                        for (int g = 0; g < 2; ++g) {
+                            const float vv[4] = {acc[4 * g][4 * h + y], acc[4 * g + 1][4 * h + y],
+                                                 acc[4 * g + 2][4 * h + y], acc[4 * g + 3][4 * h + y]};
+                            const long long eb = e0 + g * (BM / 2);
+                            if (a.vec_out) {
+                                // E % 4 == 0: a quad is inside or outside
+                                if (eb + 4 * ty < E)
+                                    *reinterpret_cast<float4 *>(col + eb + 4 * ty) =
+                                        make_float4(vv[0], vv[1], vv[2], vv[3]);
+                            } else {
+#pragma unroll
+                                for (int z = 0; z < 4; ++z)
+                                    if (eb + ty + z * S::TY < E)
+                                        col[eb + ty + z * S::TY] = vv[z];
+                            }
+                        }
+                    }
+            } else if (a.vec_out) {
+                // out[f][e][i], N % 4 == 0: four consecutive columns of one operator
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int c4 = cb * BN + h * (BN / 2) + 4 * tx;
+                    if (c4 >= a.C)
+                        continue;
+                    const int f4 = c4 / N, i4 = c4 - f4 * N;
+#pragma unroll
+                    for (int x = 0; x < 8; ++x) {
+                        const long long e = e0 + (x / 4) * (BM / 2) + 4 * ty + x % 4;
+                        if (e < E)
+                            *reinterpret_cast<float4 *>(a.out + ((size_t)f4 * E + e) * N + i4) =
+                                make_float4(acc[x][4 * h], acc[x][4 * h + 1], acc[x][4 * h + 2], acc[x][4 * h + 3]);
+                    }
+                }
+            } else {
+                // out[f][e][i], permuted columns: c, c + TX, c + 2 TX, c + 3 TX
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int y = 0; y < 4; ++y) {
+                        const int c = cb * BN + h * (BN / 2) + tx + y * S::TX;
+                        if (c >= a.C)
+                            break;
+                        const int f = c / N, i = c - f * N;
+                        float *o = a.out + ((size_t)f * E + e0 + 4 * ty) * N + i;
+#pragma unroll
+                        for (int x = 0; x < 8; ++x) {
+                            const int de = (x / 4) * (BM / 2) + x % 4;
+                            if (e0 + 4 * ty + de < E)
+                                o[de * N] = acc[x][4 * h + y];
+                        }
+                    }
+            }
         }
     }
     cp_async_wait_all();  // no copy outlives the CTA
 }
 
-size_t ks_smem_bytes(int Kp, int bm, int bk, int ubufs)
+// Column block width: the one of the compiled widths that covers C columns with the fewest
+// padded ones (the widest of equals: fewer passes over the u tile in shared memory).
+int ks_block_cols(int C, int bm)
 {
-    return sizeof(float) * ((size_t)ubufs * Kp * (bm + 4) + 2 * (size_t)bk * (kKsBN + 4));
+    if (bm != 128)
+        return 128;
+    int best = 128;
+    for (int bn : {112, 96, 80, 64})
+        if ((C + bn - 1) / bn * bn < (C + best - 1) / best * best)
+            best = bn;
+    return best;
+}
+
+int ks_threads(int bm, int bn) { return (bm / 8) * (bn / 8); }
+
+size_t ks_smem_bytes(int Kp, int bm, int bk, int bn, int ubufs)
+{
+    return sizeof(float) * ((size_t)ubufs * Kp * (bm + 4) + 2 * (size_t)bk * (bn + 4));
+}
+
+template <int LAYOUT, int BK>
+static void *ks_fn128(int bn)
+{
+    switch (bn) {
+    case 64: return reinterpret_cast<void *>(&ks_contract_kernel<LAYOUT, 128, BK, 64>);
+    case 80: return reinterpret_cast<void *>(&ks_contract_kernel<LAYOUT, 128, BK, 80>);
+    case 96: return reinterpret_cast<void *>(&ks_contract_kernel<LAYOUT, 128, BK, 96>);
+    case 112: return reinterpret_cast<void *>(&ks_contract_kernel<LAYOUT, 128, BK, 112>);
+    default: return reinterpret_cast<void *>(&ks_contract_kernel<LAYOUT, 128, BK, 128>);
+    }
 }
 
 template <int LAYOUT>
-static void *ks_fn(int bm, int bk)
+static void *ks_fn(int bm, int bk, int bn)
 {
     if (bm == 128)
-        return bk == 16 ? reinterpret_cast<void *>(&ks_contract_kernel<LAYOUT, 128, 16>)
-                        : reinterpret_cast<void *>(&ks_contract_kernel<LAYOUT, 128, 8>);
-    return bk == 16 ? reinterpret_cast<void *>(&ks_contract_kernel<LAYOUT, 64, 16>)
-                    : reinterpret_cast<void *>(&ks_contract_kernel<LAYOUT, 64, 8>);
+        return bk == 16 ? ks_fn128<LAYOUT, 16>(bn) : ks_fn128<LAYOUT, 8>(bn);
+    return bk == 16 ? reinterpret_cast<void *>(&ks_contract_kernel<LAYOUT, 64, 16, 128>)
+                    : reinterpret_cast<void *>(&ks_contract_kernel<LAYOUT, 64, 8, 128>);
 }
 
 lc_status ks_launch(const KsArgs &a, int layout, int bm, int bk, int grid, cudaStream_t s, bool set_attr)
 {
     if (!(bm == 64 || bm == 128) || !(bk == 8 || bk == 16))
         return LC_ERR_INVALID_VARIANT;
-    void *fn = layout == LC_LAYOUT_NODE_MAJOR ? ks_fn<LC_LAYOUT_NODE_MAJOR>(bm, bk) : ks_fn<LC_LAYOUT_ELEM_MAJOR>(bm, bk);
-    const size_t smem = ks_smem_bytes(a.Kp, bm, bk, a.ubufs);
+    void *fn = layout == LC_LAYOUT_NODE_MAJOR ? ks_fn<LC_LAYOUT_NODE_MAJOR>(bm, bk, a.bn)
+                                              : ks_fn<LC_LAYOUT_ELEM_MAJOR>(bm, bk, a.bn);
+    const size_t smem = ks_smem_bytes(a.Kp, bm, bk, a.bn, a.ubufs);
     cudaError_t e = cudaSuccess;
     if (set_attr) {
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -312,7 +396,7 @@ lc_status ks_launch(const KsArgs &a, int layout, int bm, int bk, int grid, cudaS
         return LC_OK;  // attribute set only (a capture launches later)
     KsArgs args = a;
     void *params[] = {&args};
-    e = cudaLaunchKernel(fn, dim3(grid), dim3(bm / 8 * 16), params, smem, s);
+    e = cudaLaunchKernel(fn, dim3(grid), dim3(ks_threads(bm, a.bn)), params, smem, s);
     return e == cudaSuccess ? LC_OK : cuda_fail(e);
 }
 

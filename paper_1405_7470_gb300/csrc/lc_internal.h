@@ -102,7 +102,7 @@ struct WarpArgs {
     int tail_free;
 };
 
-// K-split SIMT kernel (FP32): 8 x 8 register blocks over a BM x 128 output tile, the
+// K-split SIMT kernel (FP32): 8 x 8 register blocks over a BM x BN output tile, the
 // reduction over j cut into chunks of BK (split_iname on j) whose D^T slices are fetched
 // asynchronously into a two-slot ring, the u tile resident (transposed) for all column blocks.
 struct KsArgs {
@@ -112,7 +112,7 @@ struct KsArgs {
     long long E;
     int N, F, C;       // C = F * N output columns
     int Kp, nkc;       // N rounded up to the chunk width, and the number of chunks
-    int nblocks;       // column blocks of 128
+    int bn, nblocks;   // column block width (ks_block_cols) and the number of blocks
     long long ntiles;  // element tiles of BM
     int ubufs;         // u tile buffers: 2 = the next tile's u is fetched during this tile
     int vec_u;         // node-major: 16-byte copies of u rows (E % 4 == 0)
@@ -120,7 +120,9 @@ struct KsArgs {
 };
 // set_attr: set the instance's shared-memory size first; grid <= 0: only that.
 lc_status ks_launch(const KsArgs &a, int layout, int bm, int bk, int grid, cudaStream_t s, bool set_attr = true);
-size_t ks_smem_bytes(int Kp, int bm, int bk, int ubufs);
+size_t ks_smem_bytes(int Kp, int bm, int bk, int bn, int ubufs);
+int ks_block_cols(int C, int bm);
+int ks_threads(int bm, int bn);
 
 // Tensor-core kernel (tcgen05): one column block of G operators per CTA.
 struct TcArgs {
