@@ -127,14 +127,13 @@ struct lc_variant {
                                  tensor-core engine: operators per CTA column block (0 = most) */
     int32_t unroll;           /* unr tag on the j reduction: 1, 2, 4 or 8; tensor-core engine:
                                  epilogue threads per tile row, 1 to 4 (conversion threads per
-                                 row: the same, 2 for 4) */
+                                 row: 1; 2 to 4, growing with N; 3; 2) */
     int32_t prefetch_smem;    /* add_prefetch of the u tile into shared memory by TMA (1) or
                                  direct global loads into registers (0); tensor-core engine: 1,
-                                 or 2 = each converting thread takes its values into registers,
-                                 splits them into their bf16 terms and frees the stage at once,
-                                 so only its stores wait for the A buffer (K of one block, at
-                                 most 3 chunks of 8 nodes a thread for BF16, 2 for BF16X3;
-                                 others take the plain path) */
+                                 or 2 = each converting thread takes all its values into
+                                 registers and frees the stage at once, before it waits for
+                                 the A buffer (at most 3 chunks of 8 nodes a thread; others
+                                 take the plain path) */
     int32_t tail_free;        /* 1: no guard on the last e tile; only accepted when an
                                  assumption "E mod m = 0" with m a multiple of tile_e holds */
     int32_t stages;           /* u tiles in flight in shared memory (TMA ring depth), >= 1 */
@@ -159,9 +158,10 @@ struct lc_variant {
                                  operand) lives: 0 = the planner's choice, 1 = shared memory,
                                  2 = tensor memory beside the accumulators, written by the
                                  conversion warps with tcgen05.st: frees shared memory and its
-                                 bandwidth (BF16X3: one accumulator region per buffer, the
-                                 products unstacked; the planner takes it where no shared-
-                                 memory plan fits, N up to 128; not for the three-term
+                                 bandwidth (BF16X3: the products stacked where two accumulators
+                                 and the A terms fit tensor memory, one operator up to N = 88,
+                                 unless mma_order is 2; else one accumulator region per buffer,
+                                 N up to 128; not for the three-term
                                  geometric-factor kernel) */
 };
 
@@ -169,8 +169,8 @@ struct lc_variant {
  * A reasonable descriptor for (E, N, F, layout, precision): fills *v.  The choices follow
  * the autotuner's measurements on this GPU: FP32 on the warp engine up to N = 12, SIMT
  * tiles below N = 64, the K-split engine from N = 64; BF16 and BF16X3 on the tensor cores
- * (BF16X3 with the A terms in shared memory, from about N = 100 to 128 in tensor memory),
- * and where no tensor-core plan exists the FP32 kernels, whose error is below both
+ * (BF16X3 with the A terms in shared memory or, where that is faster, in tensor memory, up
+ * to N = 128), and where no tensor-core plan exists the FP32 kernels, whose error is below both
  * reduced-precision bounds; FP64 SIMT tiles.  No GPU work is done.
  * Errors: LC_ERR_INVALID_ARGUMENT, LC_ERR_UNSUPPORTED (no engine supports it).
  */
@@ -421,9 +421,12 @@ lc_status lc_grouped_workspace_size(const lc_kernel *k, const lc_variant *v, con
  * a tensor-core plan (lc_variant_validate's rules; the epilogue works in 8-column chunks)
  * for the variant, or else for the first of its changes "stages = 1", "the other K-block
  * width (elems_per_thread 1 <-> 64)", "store_rows = 32" (element-major) and their
- * combinations, with the same CTA size (unroll), runs in one tensor-core launch, one CTA per SM at most: every (group,
- * column block) unit gets at least one CTA, and the rest go to the unit whose estimated
- * time (tiles x per-tile cost / CTAs) is the largest.  More units than SMs is
+ * combinations, with the same CTA size (unroll), runs in one tensor-core launch, one CTA
+ * per SM at most: every (group, column block) unit gets at least one CTA, and the rest go to
+ * the unit whose estimated time (tiles x per-tile cost / CTAs) is the largest.  A group that
+ * would hold the whole GPU for more than about 30 us runs after it as a launch of its own with
+ * the library's default descriptor (unless the variant sets split_i, mma_order, a_operand or
+ * max_ctas).  More units than SMs is
  * LC_ERR_INVALID_VARIANT.  Groups without a tensor-core plan (e.g. N above the plans'
  * limit) run after it, each in a K-split FP32 launch (tiles of 128 elements, j chunks of 16,
  * one u buffer), or, without a K-split plan, in a FP32 SIMT grouped launch (8 x 8 register

@@ -1185,7 +1185,11 @@ static lc_status resolve(const Kernel &K, long long E, int N, int F, const lc_va
         t.stages = v->stages;
         t.early_release = v->prefetch_smem == 2;
         t.threads_per_row = v->unroll;
-        t.conv_threads_per_row = std::min(v->unroll, 6 - v->unroll);
+        // two epilogue threads a row: as many conversion threads as bring a thread's share of the
+        // row down to three chunks of 8 nodes, 2 to 4 (N = 35: 2, N = 84: 4); else as many as
+        // epilogue threads, 26 warps in all
+        t.conv_threads_per_row = v->unroll == 2 ? std::max(2, std::min(4, ((N + 7) / 8 + 2) / 3))
+                                                : std::min(v->unroll, 6 - v->unroll);
         const size_t W = 2 * (size_t)t.KB;
         // rows per element-major bulk store: whole tiles of every operator of the block for
         // small N (few, large stores), else 32-row pieces of one operator at a time (the
@@ -1199,32 +1203,44 @@ static lc_status resolve(const Kernel &K, long long E, int N, int F, const lc_va
             // the BF16X3 terms stack (2 CBp <= 256) or the block fit (CBp <= 256) at all
             auto cbp = [&](int np) { return (G * np + 15) / 16 * 16; };
             const int np16 = (N + 15) / 16 * 16, np8 = (N + 7) / 8 * 8;
-            const bool want_stack = NT == 3 && v->mma_order != 2 && !a_tm;
+            bool want_stack = NT == 3 && v->mma_order != 2 && !a_tm;
+            // the A terms in tensor memory, stacked: regions CBs = CB rounded up to 8 columns apart
+            // (the last product's MMA writes CBp - CBs columns more), so that two accumulators and
+            // three A terms fit the 512 columns up to N = 88 with one operator
+            const int cbs8 = (G * np8 + 7) / 8 * 8;
+            q.a_cols = a_tm ? NT * q.Kt / 2 : 0;
+            const bool tm_stack = a_tm && NT == 3 && v->mma_order == 0 && 2 * cbs8 <= 256 &&
+                                  2 * (cbs8 + cbp(np8)) + q.abufs * q.a_cols <= 512;
             if (want_stack && 2 * cbp(np16) > 256 && 2 * cbp(np8) <= 256)
                 q.Np = np8;
-            else if ((NT == 3 || a_tm) && !want_stack && cbp(np8) < cbp(np16))
-                q.Np = np8;  // one accumulator region: the narrowest padding (smaller B, fewer columns)
+            else if (tm_stack || ((NT == 3 || a_tm) && !want_stack && cbp(np8) < cbp(np16)))
+                q.Np = np8;  // the narrowest padding (smaller B, fewer columns)
             else
                 q.Np = cbp(np16) <= 256 ? np16 : np8;
+            want_stack = want_stack || tm_stack;
             // three terms, whole-tile epilogue (node-major, or element-major stores of whole
             // tiles): the operators packed without padding where that narrows the MMAs, whose
             // time grows with their N (the epilogue chunks may then cross an operator's end)
             if (NT == 3 && !geo && (node || t.store_quarters == 4) && N >= 8 && cbp(N) < cbp(q.Np) &&
                 (!want_stack || 2 * cbp(N) <= 256))
                 q.Np = N;
-            q.chunk = q.Np % 16 == 0 && !geo ? 16 : 8;
+            q.chunk = (q.Np % 16 == 0 || (node && q.Np == N)) && !geo ? 16 : 8;
             q.CB = G * q.Np;
             q.CBp = cbp(q.Np);
             if (q.CBp > 256)
                 return false;
-            q.stack = want_stack && 2 * q.CBp <= 256;
+            q.CBs = tm_stack ? (q.CB + 7) / 8 * 8 : q.CBp;
+            q.stack = want_stack && 2 * q.CBs <= 256;
             if (v->mma_order == 1 && !q.stack)
                 return false;  // the stacked order needs 2 x MMA N <= 256
-            q.tmem_cols = 32;
-            while (q.tmem_cols < (q.stack ? 2 : 1) * q.CBp)
-                q.tmem_cols *= 2;
+            if (tm_stack) {
+                q.tmem_cols = q.CBs + q.CBp;
+            } else {
+                q.tmem_cols = 32;
+                while (q.tmem_cols < (q.stack ? 2 : 1) * q.CBp)
+                    q.tmem_cols *= 2;
+            }
             q.a_tmem = a_tm;
-            q.a_cols = a_tm ? NT * q.Kt / 2 : 0;
             const int need = 2 * q.tmem_cols + q.abufs * q.a_cols;
             if (need > 512)
                 return false;
@@ -1232,7 +1248,7 @@ static lc_status resolve(const Kernel &K, long long E, int N, int F, const lc_va
             while (q.tmem_alloc < need)
                 q.tmem_alloc *= 2;
             size_t off = 0;
-            off += (size_t)NT * q.nkb * q.CBp * W;                       // B terms
+            off += (size_t)q.nkb * (NT * q.CBs + q.CBp - q.CBs) * W;     // B terms
             off += a_tm ? 0 : (size_t)q.abufs * NT * q.nkb * 128 * W;  // A terms
             q.off_stage = (unsigned)off;
             off += (size_t)q.stages * 128 * N * 4;
@@ -1267,17 +1283,20 @@ static lc_status resolve(const Kernel &K, long long E, int N, int F, const lc_va
                 const bool a_tm = tm_first ? pass == 0 : pass == 1;
                 if ((a_tm && v->a_operand == 1) || (!a_tm && v->a_operand == 2) || (a_tm && geo && NT != 1))
                     continue;
-                for (int c = 0; c < ncombos && !found; ++c) {
-                    TcArgs q = t;
-                    q.obufs = node ? 1 : combos[c][0];
-                    q.abufs = combos[c][1];
-                    if (!node && v->out_buffers && q.obufs != v->out_buffers)
-                        continue;
-                    if (plan(g, q, a_tm)) {
-                        t = q;
-                        found = true;
+                // three terms in tensor memory: a stacked plan before any buffer count (it keeps
+                // the large products apart, which is the more accurate order)
+                for (int stacked = (a_tm && NT == 3) ? 1 : 0; stacked >= 0 && !found; --stacked)
+                    for (int c = 0; c < ncombos && !found; ++c) {
+                        TcArgs q = t;
+                        q.obufs = node ? 1 : combos[c][0];
+                        q.abufs = combos[c][1];
+                        if (!node && v->out_buffers && q.obufs != v->out_buffers)
+                            continue;
+                        if (plan(g, q, a_tm) && (!stacked || q.stack)) {
+                            t = q;
+                            found = true;
+                        }
                     }
-                }
         }
         if (!found)
             return LC_ERR_INVALID_VARIANT;
@@ -1902,49 +1921,98 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
         d.engine = LC_ENGINE_TCGEN05;
         d.tile_e = 128;
         d.split_i = 0;
-        d.unroll = 4;
-        // BF16X3: three epilogue and conversion threads per row with the stage released early
-        // (element-major), two with two stages (node-major): the fastest measured at N = 35
-        // 64-wide K-blocks first: a tcgen05.mma reading 128-byte swizzled rows costs the
-        // fewest cycles; then the narrowest blocks that cover K (least shared memory).
-        // BF16X3: the A terms in shared memory first (the stacked order), one stage first (two
-        // stages leave room for one output slot only); BF16: the planner's placement, two stages.
-        const bool x3 = precision == LC_PREC_BF16X3;
+        const bool x3 = precision == LC_PREC_BF16X3, node = layout == LC_LAYOUT_NODE_MAJOR;
+        const bool geo = kh->k.kind == KIND_GEO;
         lc_status st = LC_ERR_INVALID_VARIANT;
-        const bool x3node = x3 && layout == LC_LAYOUT_NODE_MAJOR;
-        if (x3) {
-            d.unroll = x3node ? 2 : 3;
-            d.prefetch_smem = x3node ? 1 : 2;
+        Resolved r;
+        // The candidates come in the order a sweep of descriptors found them fastest (N = 6 to
+        // 120, F = 1 to 4); the first whose plan fits (and, where asked, has two A buffers,
+        // two output slots or every operator in one block) is taken.
+        auto take = [&](int unroll, int prefetch, int stages, int kbw, int rows, int aop, int split, auto &&good) {
+            if (st != LC_ERR_INVALID_VARIANT)
+                return;
+            lc_variant c = d;
+            c.unroll = unroll;
+            c.prefetch_smem = prefetch;
+            c.stages = stages;
+            c.elems_per_thread = kbw;
+            c.store_rows = node ? 0 : rows;
+            c.a_operand = aop;
+            c.split_i = split;
+            const lc_status rs = resolve(kh->k, E, N, F, &c, r, false);
+            if (rs == LC_OK && good(r.tc))
+                d = c;
+            if (rs != LC_OK || good(r.tc))
+                st = rs;
+        };
+        auto any = [](const TcArgs &) { return true; };
+        auto roomy = [](const TcArgs &t) { return t.abufs == 2 && t.obufs >= 2; };
+        auto all_ops = [F](const TcArgs &t) { return t.G == F; };
+        // (three terms with A in tensor memory: only with the large products kept apart, whose
+        // error is 8 to 60 % below the one-region order's)
+        auto stacked = [](const TcArgs &t) { return t.stack != 0; };
+        auto stacked_all = [F](const TcArgs &t) { return t.stack && t.G == F && t.obufs >= 2; };
+        auto slots2 = [F](const TcArgs &t) { return t.G == F && t.obufs >= 2; };
+        if (x3 && node) {
+            // few warps (one thread a row and role: 352 threads) and deep staging: N = 35, F = 3,
+            // E = 2^20 102 us against 114 with 608 threads and two stages; geometric factors
+            // need more epilogue threads (139 against 158 us)
+            const int u = geo ? 3 : (N > 48 && N <= 64 ? 2 : 1);
+            for (int stg : {3, 2, 1})
+                for (int kbw : {64, 1})
+                    take(u, 1, stg, kbw, 0, 1, 0, any);
+        } else if (x3 && N <= 48) {
+            // whole-tile stores; two A buffers and two slots beside three stages where they fit
+            // (N = 20, F = 3, E = 2^20: 62 us against 101 with one stage); else the A terms in
+            // tensor memory where that keeps every operator in one block (N = 35, F = 2, E =
+            // 2^18: 25 against 34); else narrow K-blocks (N = 35, F = 3, E = 2^20: 104 against
+            // 127); else tensor memory with fewer operators (N = 48, F = 4, E = 2^18: 58 against 104)
+            take(geo ? 4 : 3, 1, 3, 64, 128, 1, 0, roomy);
+            if (!geo)
+                for (int stg : {3, 2})
+                    take(3, 1, stg, 64, 128, 2, 0, stacked_all);
+            for (int stg : {3, 2})
+                take(geo ? 3 : 4, stg == 2 ? 2 : 1, stg, 1, 128, 1, 0, slots2);
+            if (!geo)
+                for (int split : {0, (F + 1) / 2})
+                    for (int stg : {3, 2})
+                        take(3, 1, stg, 64, 128, 2, split, stacked);
+        } else if (x3 && !geo && N <= 88) {
+            // every operator in one block from shared memory up to N = 64 (N = 56, F = 3, E =
+            // 2^19: 95 us against 109); else one operator per block, the A terms in tensor
+            // memory: shared memory's bandwidth bounds these sizes, and A's stores and reads
+            // are over a third of its traffic (N = 84, F = 4, E = 2^20: 410 us, 470 with A in
+            // shared memory)
+            if (N <= 64 && F > 1)
+                for (int stg : {2, 1})
+                    take(2, 2, stg, 1, 32, 1, 0, all_ops);
+            for (int stg : {3, 2, 1})
+                take(2, 1, stg, 64, N > 80 ? 32 : 128, 2, 1, stacked);
+        } else if (!x3 && !node) {
+            // BF16: many warps up to N = 48 (N = 35, F = 3, E = 2^20: 99 us), fewer above (N = 120,
+            // F = 3, E = 2^18: 92 against 105)
+            const int u = N <= 48 ? 3 : 2;
+            for (int stg : {2, 3, 1})
+                for (int kbw : {64, 1})
+                    take(u, 1, stg, N > 96 ? 65 - kbw : kbw, 0, 0, 0, any);
+        } else if (!x3) {
+            // BF16, node-major: N = 35, F = 3, E = 2^20 99 us (111 with two stages); N = 84, F = 4,
+            // E = 2^19 168 (177)
+            const int u = N <= 64 ? 3 : 1;
+            for (int stg : {3, 2, 1})
+                for (int kbw : {64, 1})
+                    take(u, 1, stg, kbw, 0, 0, 0, any);
         }
-        for (int aop : {x3 ? 1 : 0})
-            for (int kbw : {64, 1})
-                for (int stg : {x3 && !x3node ? 1 : 2, x3 && !x3node ? 2 : 3, 1}) {
-                    if (st == LC_OK)
-                        break;
-                    d.a_operand = aop;
-                    d.elems_per_thread = kbw;
-                    d.stages = stg;
-                    st = lc_variant_validate(kh, E, N, F, &d);
-                    if (st != LC_OK && st != LC_ERR_INVALID_VARIANT)
-                        return st;
-                }
-        if (st != LC_OK && x3) {
-            // no shared-memory plan for the three A terms (N of about 100 and more): the
-            // planner's placement (tensor memory), one operator per column block, 32-row
-            // stores; measured at N = 120, E = 310977: 0.44 ms against 0.69 ms for the K-split
-            // FP32 kernel (node-major 0.65 against 0.89 ms)
-            d.a_operand = 0;
-            d.split_i = 1;
-            d.unroll = 3;
-            d.prefetch_smem = 1;
-            d.stages = 1;
-            d.store_rows = layout == LC_LAYOUT_ELEM_MAJOR ? 32 : 0;
-            for (int kbw : {64, 1}) {
-                d.elems_per_thread = kbw;
-                st = lc_variant_validate(kh, E, N, F, &d);
-                if (st == LC_OK || st != LC_ERR_INVALID_VARIANT)
-                    break;
-            }
+        if (x3) {
+            // the rest in shared memory, then (N of about 100 and more) A in tensor memory, one
+            // operator per column block, 32-row stores: N = 120, F = 3, E = 2^18 217 us against
+            // 0.58 ms for the K-split FP32 kernel
+            for (int stg : {1, 2})
+                for (int kbw : {64, 1})
+                    take(geo && !node ? 3 : 2, 1, stg, kbw, 0, 1, 0, any);
+            for (int stg : {2, 1})
+                for (int kbw : {64, 1})
+                    take(2, 1, stg, kbw, 32, 0, 1, any);
         }
         if (st == LC_OK) {
             *v = d;
@@ -2265,11 +2333,13 @@ struct KsLaunch {
     int grid, bm, bk, group;
 };
 
-// One plain tensor-core launch: a group of a tensor-core grouped plan whose plan needs the A
-// terms in tensor memory (no shared-memory plan fits), which the grouped kernel does not take.
+// One plain tensor-core launch of a tensor-core grouped plan: a large group with its own default
+// descriptor, or a group whose plan needs the A terms in tensor memory (no shared-memory plan
+// fits), which the grouped kernel does not take.
 struct TcLaunch {
     TcArgs a;
     int layout, nterms, grid, group;
+    lc_variant v;
 };
 
 }  // namespace lc
@@ -2524,7 +2594,24 @@ struct GroupedPlanTc {
     int grid = 0, threads = 0, nterms = 1;
     size_t smem = 0;
     std::vector<int> tc_groups, simt_groups;
+    std::vector<int> own_groups;  // large groups that run as a launch of their own default descriptor (gv)
 };
+
+// Estimated seconds of a group's tile and column block in the grouped launch: its HBM bytes at the
+// SM's share of the copy rate (0.8 efficiency), or the MMA chain at about 120 cycles an
+// instruction, plus a fixed pipeline cost.
+static double grouped_tile_cost(const TcArgs &t, int nterms, int gb, int sms)
+{
+    const int mmas = (nterms == 1 ? 1 : (t.stack ? 5 : 6)) * (t.Kt / 16);
+    const double bytes = 128.0 * t.N * 4.0 * (1 + gb);
+    return std::max(bytes / (6.7e12 / sms) / 0.8, mmas * 120.0 / 1.9e9) + 4e-7;
+}
+
+// A group that would hold the whole GPU this long runs as its own launch, with the library's
+// default descriptor for it: the grouped launch gives every group one CTA size, 8-column
+// epilogue chunks and a shared-memory plan (N = 84, F = 3, E = 1373370: 0.62 ms in it, 0.41 ms
+// alone), while a launch costs about 6 us.
+static constexpr double kOwnLaunchSeconds = 3e-5;
 
 static lc_status grouped_plan_tc(const Kernel &K, const lc_variant *v, const lc_group *groups, int ng,
                                  GroupedPlanTc &T)
@@ -2586,25 +2673,38 @@ static lc_status grouped_plan_tc(const Kernel &K, const lc_variant *v, const lc_
         }
         T.gv[gi] = vg;
         TcArgs t = r.tc;
+        double whole = 0;  // the group's time on the whole GPU
+        for (int b = 0; b < t.nblocks; ++b)
+            whole += t.ntiles * grouped_tile_cost(t, T.nterms, std::min(t.G, G.F - b * t.G), sms) / sms;
+        // (a variant that fixes how the products are formed or bounds the grid is kept as given)
+        if (whole > kOwnLaunchSeconds && v->mma_order == 0 && v->a_operand == 0 && v->split_i == 0 &&
+            v->max_ctas == 0) {
+            const lc_kernel kh{K};
+            lc_variant dv;
+            Resolved dr;
+            if (lc_variant_default(&kh, G.E, G.N, G.F, v->layout, v->precision, &dv) == LC_OK &&
+                dv.engine == LC_ENGINE_TCGEN05 && resolve(K, G.E, G.N, G.F, &dv, dr, true) == LC_OK &&
+                (dr.tc.stack || !t.stack)) {
+                T.gv[gi] = dv;
+                T.own_groups.push_back(gi);
+                continue;
+            }
+        }
         t.D = static_cast<const float *>(G.D_dev);
         t.u = static_cast<const float *>(G.u_dev);
         t.out = static_cast<float *>(G.out_dev);
         t.r = nullptr;
         t.err = error_word();
         t.chunk = 8;  // one kernel instance for all groups: 8-column epilogue chunks
+        t.conv_threads_per_row = std::min(v->unroll, 6 - v->unroll);  // and one CTA size
         const int tg = (int)T.tc_groups.size();
         T.P.g[tg] = t;
         T.tc_groups.push_back(gi);
         T.smem = std::max(T.smem, (size_t)t.smem_bytes);
         T.threads = tc_threads(t);
-        // per tile: its HBM bytes at the SM's share of the copy rate (0.6 efficiency), or the
-        // MMA chain at about 300 cycles an instruction, plus a fixed pipeline cost
-        const int kn = t.Kt;
-        const int mmas = (T.nterms == 1 ? 1 : (t.stack ? 5 : 6)) * (kn / 16);
         for (int b = 0; b < t.nblocks; ++b) {
             const int gb = std::min(t.G, G.F - b * t.G);
-            const double bytes = 128.0 * G.N * 4.0 * (1 + gb);
-            const double cost = std::max(bytes / (6.7e12 / sms) / 0.6, mmas * 300.0 / 1.9e9) + 4e-7;
+            const double cost = grouped_tile_cost(t, T.nterms, gb, sms);
             units.push_back({tg, b, t.ntiles, cost});
         }
     }
@@ -2710,7 +2810,7 @@ static lc_variant grouped_tc_fallback(const lc_variant *v)
     s.tile_e = 128;
     s.elems_per_thread = 64;
     s.split_i = 1;
-    s.unroll = 3;
+    s.unroll = 2;
     s.prefetch_smem = 1;
     s.stages = 1;
     s.store_rows = v->layout == LC_LAYOUT_ELEM_MAJOR ? 32 : 0;
@@ -2791,29 +2891,41 @@ static lc_status grouped_plan_all(const Kernel &K, const lc_variant *v, const lc
     // grouped launch
     A.ks_v = grouped_ks_fallback(v);
     A.tcl_v = grouped_tc_fallback(v);
+    auto add_tc = [&](int gi, const lc_variant &tv) -> lc_status {
+        const lc_group &G = groups[gi];
+        Resolved r;
+        const lc_status rs = resolve(K, G.E, G.N, G.F, &tv, r, true);
+        if (rs != LC_OK)
+            return rs;
+        TcLaunch L;
+        L.a = r.tc;
+        L.a.D = static_cast<const float *>(G.D_dev);
+        L.a.u = static_cast<const float *>(G.u_dev);
+        L.a.out = static_cast<float *>(G.out_dev);
+        L.a.err = error_word();
+        L.layout = r.layout;
+        L.nterms = A.T.nterms;
+        L.grid = r.tc_grid;
+        L.group = gi;
+        L.v = tv;
+        A.tcl.push_back(L);
+        return LC_OK;
+    };
+    for (int gi : A.T.own_groups) {
+        st = add_tc(gi, A.T.gv[gi]);
+        if (st != LC_OK)
+            return st;
+    }
     for (int gi : A.T.simt_groups) {
         const lc_group &G = groups[gi];
         if (G.E == 0)
             continue;
         if (v->precision == LC_PREC_BF16X3) {
-            Resolved r;
-            const lc_status rs = resolve(K, G.E, G.N, G.F, &A.tcl_v, r, true);
+            const lc_status rs = add_tc(gi, A.tcl_v);
             if (rs == LC_ERR_NO_DEVICE || rs == LC_ERR_CUDA)
                 return rs;
-            if (rs == LC_OK) {
-                TcLaunch L;
-                L.a = r.tc;
-                L.a.D = static_cast<const float *>(G.D_dev);
-                L.a.u = static_cast<const float *>(G.u_dev);
-                L.a.out = static_cast<float *>(G.out_dev);
-                L.a.err = error_word();
-                L.layout = r.layout;
-                L.nterms = 3;
-                L.grid = r.tc_grid;
-                L.group = gi;
-                A.tcl.push_back(L);
+            if (rs == LC_OK)
                 continue;
-            }
         }
         bool added = false;
         const lc_status sk = grouped_add_ks(K, A.ks_v, G, gi, A.ks, &added);
@@ -2953,9 +3065,11 @@ lc_status lc_grouped_plan_create(const lc_kernel *kh, const lc_variant *v, const
     for (const KsLaunch &L : A.ks)
         plan->group_variant[L.group] = A.ks_v;
     for (const TcLaunch &L : A.tcl)
-        plan->group_variant[L.group] = A.tcl_v;
+        plan->group_variant[L.group] = L.v;
     plan->ks = A.ks;
     plan->tcl = A.tcl;
+    for (const TcLaunch &L : A.tcl)
+        plan->nsegs += L.grid;
     plan->layout = v->layout;
     // shared-memory sizes, before any capture
     for (const KsLaunch &L : A.ks) {

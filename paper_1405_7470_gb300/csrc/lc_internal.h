@@ -137,10 +137,14 @@ struct TcArgs {
     int Np;         // accumulator columns per operator: N rounded up to 16 (or to 8)
     int chunk;      // epilogue chunk: 16 columns when Np is a multiple of 16, else 8
     int CB, CBp;    // columns per block (G * Np) and the MMA N (CB rounded up to 16)
+    int CBs;        // columns between the terms of B and between the regions of a stacked
+                    // accumulator: CBp, or CB rounded up to 8 (A in tensor memory, stacked: two
+                    // accumulators and the three A terms must fit its 512 columns)
     int Kp, KB, nkb;  // K padded to the block width, K-block width (16/32/64 -> 32/64/128-byte swizzle), blocks
     int Kt;         // K the MMAs read: N rounded up to 16 (zeros past N)
-    int stack;      // BF16X3 with two B terms stacked along N (2 * CBp <= 256): 5 MMAs per K step, not 6
-    int tmem_cols;  // columns per accumulator (power of two >= CBp, or >= 2 * CBp when stacked)
+    int stack;      // BF16X3 with two B terms stacked along N (2 * CBs <= 256): 5 MMAs per K step, not 6
+    int tmem_cols;  // columns per accumulator (power of two >= CBp, or >= 2 * CBp when stacked; CBs + CBp
+                    // when stacked with A in tensor memory)
     int a_tmem;     // 1: the A terms live in tensor memory after the two accumulators
     int a_cols;     // tensor-memory columns per A buffer (NT terms x K/2 packed bf16 pairs)
     int tmem_alloc; // tensor-memory columns allocated (power of two >= 32)

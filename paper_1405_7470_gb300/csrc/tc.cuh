@@ -31,6 +31,14 @@
 //                  along e);
 //   store warp     issues the bulk stores of the whole-tile slots and hands each slot
 //                  back once the copies have read it (idle in the other layouts).
+// What bounds it: shared memory's bandwidth (128 B a clock) for one operator of N = 84, where
+// per tile and operator the MMAs read 960 clocks of A and 860 of B, the conversion stores 530 of
+// A and loads 350 of u, and the output passes through twice (680): A in tensor memory takes a
+// third of it away (E = 2^20, F = 4, three terms: 470 -> 413 us, HBM floor 263).  For N = 35,
+// F = 3 the HBM rate is close (191 us at E = 2^21, floor 175; 253 before the epilogue, the
+// conversion and the MMA issue were cut to what they need: no integer divisions, chunk
+// offsets from a table, 16-byte reads where rows allow them, 32-bit descriptors).
+//
 // Setup: the MMA warp allocates the accumulators; all threads split D into the
 // B-operand terms, resident for the CTA's lifetime.
 // Every mbarrier wait is bounded in time; on a timeout the kernel sets the device
@@ -39,6 +47,8 @@
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "lc_internal.h"
 #include "tma.cuh"
@@ -238,15 +248,58 @@ __device__ __forceinline__ bool bar_or(int id, int nthreads, bool v)
     }
 }
 
+// A position in a ring of `n` buffers and its phase parity, advanced without divisions (one
+// integer division per ring, role and tile was a third of the instructions the kernel issued).
+struct Ring {
+    int i = 0;
+    uint32_t ph = 0;
+    __device__ __forceinline__ void next(int n)
+    {
+        if (++i == n) {
+            i = 0;
+            ph ^= 1u;
+        }
+    }
+};
+
 // K-blocks per A buffer with their own full/empty barrier pair
 static constexpr int kTcMaxKB = 16;
 
-// Accumulator chunks (CW columns each) an epilogue warp loads before one wait: 32 registers
-// of loaded values, half of them per region when the BF16X3 terms are stacked.
+// Accumulator chunks (CW columns each) an epilogue warp loads before one wait.  A load and its
+// wait take 25 (8 columns) to 40 cycles (16), so one chunk at a time costs little, and the
+// registers of a second one (of both regions, with stacked BF16X3 terms) would spill.
 template <int NT, int CW>
 struct EpiBatch {
-    static constexpr int value = (NT == 3 ? 16 : 32) / CW;
+    static constexpr int value = NT == 3 ? 1 : 32 / CW;
 };
+
+// r += r2, column by column (both accumulator regions of stacked BF16X3 terms), two per instruction
+template <int CW>
+__device__ __forceinline__ void add_regions(uint32_t *r, const uint32_t *r2)
+{
+#pragma unroll
+    for (int q = 0; q < CW; q += 2) {
+        asm("{\n.reg .b64 x, y;\nmov.b64 x, {%0, %1};\nmov.b64 y, {%2, %3};\nadd.rn.f32x2 x, x, y;\n"
+            "mov.b64 {%0, %1}, x;\n}\n"
+            : "+r"(r[q]), "+r"(r[q + 1])
+            : "r"(r2[q]), "r"(r2[q + 1]));
+    }
+}
+
+// CW consecutive values to shared memory; vec: o is 16-byte aligned
+template <int CW>
+__device__ __forceinline__ void store_chunk(float *o, const uint32_t *r, bool vec)
+{
+    if (vec) {
+#pragma unroll
+        for (int h = 0; h < CW / 4; ++h)
+            *reinterpret_cast<uint4 *>(o + 4 * h) = make_uint4(r[4 * h], r[4 * h + 1], r[4 * h + 2], r[4 * h + 3]);
+    } else {
+#pragma unroll
+        for (int q = 0; q < CW; ++q)
+            o[q] = __uint_as_float(r[q]);
+    }
+}
 
 template <int CW>
 __device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t *r)
@@ -277,7 +330,7 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
     unsigned char *smem = smem_dyn + (((raw + 1023u) & ~1023u) - raw);
     const uint32_t sbase = smem_addr(smem);
 
-    const int N = a.N, G = a.G, CBp = a.CBp, KB = a.KB, nkb = a.nkb;
+    const int N = a.N, G = a.G, CBp = a.CBp, CBs = a.CBs, KB = a.KB, nkb = a.nkb;
     // The A terms in tensor memory are compiled into the BF16 instances and into separate
     // three-term instances (ATM): in the three-term instances for shared-memory A, the
     // warp-uniform conversion loops the tensor-memory stores need measured slower, and with
@@ -294,7 +347,10 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
     const int W = 2 * KB;  // bytes per row of a K-block
     const long long E = a.E;
     const int S = a.stages, NA = a.abufs;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    // warp-uniform as the compiler sees it, like tmem_base below: the issue loops then keep their
+    // addresses in uniform registers
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const int He = a.threads_per_row, Hc = a.conv_threads_per_row;  // threads per tile row per role
     const int NW = 4 * He, NC = 4 * Hc;  // epilogue warps 0..NW-1, conversion warps NW..NW+NC-1
     const int row = 32 * (warp & 3) + lane;  // tile row (== TMEM lane for epilogue warps)
@@ -302,8 +358,9 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
     const int f0 = blk * G;
     const int Gb = min(G, a.F - f0);  // operators in this block
 
-    // B: per K-block, the NT terms of D^T stacked along rows (term t, column n -> row t*CBp + n)
-    const uint32_t bkb = (uint32_t)NT * CBp * W;  // bytes per K-block of B
+    // B: per K-block, the NT terms of D^T stacked along rows (term t, column n -> row t*CBs + n),
+    // then CBp - CBs rows of zeros: an MMA of N = CBp reads past its term's CBs rows
+    const uint32_t bkb = (uint32_t)(NT * CBs + CBp - CBs) * W;  // bytes per K-block of B
     const uint32_t offA = (uint32_t)nkb * bkb;
     const uint32_t termA = (uint32_t)nkb * TE * W;  // bytes per A term
     const uint32_t bufA = NT * termA;               // bytes per A buffer
@@ -317,6 +374,10 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
     uint64_t *a_full = bar + 16, *a_empty = bar + 16 + 2 * kTcMaxKB;
     // element-major whole-tile staging slots handed between the epilogue and the store warp
     uint64_t *slot_full = bar + 16 + 4 * kTcMaxKB, *slot_empty = slot_full + 4;
+    // per accumulator chunk of CW columns (at most 256 / 8): {where its first column goes, nodes from
+    // that column to its operator's end}; where = f * TE * N + i in the staged tile (element-major)
+    // or the output row f * N + i (node-major)
+    int2 *chunk_tab = reinterpret_cast<int2 *>(slot_empty + 4);
 
     const int prod_warp = NW + NC, mma_warp = NW + NC + 1, store_warp = NW + NC + 2;
     if (warp == mma_warp)
@@ -342,6 +403,11 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
         fence_mbar_init();
     }
 
+    if (tid < CBp / CW) {
+        const int c = tid * CW, fl = c / Np, i = c - fl * Np;
+        chunk_tab[tid] = make_int2(fl * (NODE ? N : TE * N) + i, N - i);
+    }
+
     // B terms: column n = f_local*Np + i of this block (i < N), K index = j; zero padding.
     {
         const int c8n = Kn / 8;
@@ -360,7 +426,8 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
             const int kb = (c8 * 8) / KB, ch = ((c8 * 8) % KB) / 8;
 #pragma unroll
             for (int tt = 0; tt < NT; ++tt)
-                *reinterpret_cast<uint4 *>(smem + (uint32_t)kb * bkb + swz_off(tt * CBp + n, ch, W)) = t[tt];
+                if (n < CBs || tt == NT - 1)
+                    *reinterpret_cast<uint4 *>(smem + (uint32_t)kb * bkb + swz_off(tt * CBs + n, ch, W)) = t[tt];
         }
         // A chunks past the last node (all zeros in every tile) are written once here; the
         // conversion warps skip them
@@ -383,7 +450,7 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_holder;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_holder, 0);
 
     // bulk-copy bytes of u tile t (0: not fetchable by the bulk engine, read from global)
     auto tile_bulk_bytes = [&](long long t) -> uint32_t {
@@ -400,11 +467,10 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
 
     if (warp == prod_warp) {
         // ---------------- producer: u tiles into the stage ring
-        int k = 0;
-        for (long long t = my_first; t < a.ntiles; t += my_step, ++k) {
-            const int s = k % S;
-            const uint32_t n = (uint32_t)(k / S);
-            if (!mbar_wait(&u_empty[s], (n & 1u) ^ 1u)) {
+        Ring us;
+        for (long long t = my_first; t < a.ntiles; t += my_step, us.next(S)) {
+            const int s = us.i;
+            if (!mbar_wait(&u_empty[s], us.ph ^ 1u)) {
                 if (lane == 0)
                     fail();
                 break;
@@ -435,40 +501,52 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
         // multiplied.  Unstacked BF16X3: products outermost, small ones first over all of K
         // (the large hh sum is accumulated last); a block is handed back after its last
         // product.
-        const uint32_t idesc = instr_desc(CBp), idesc2 = instr_desc(2 * CBp);
+        const uint32_t idesc = instr_desc(CBp), idesc2 = instr_desc(2 * CBs);
         // the K steps of block kb of one product: A term `at` times the B rows from `brow`,
         // into accumulator columns dcol.. (a descriptor advances by byte offset / 16)
         // A in tensor memory: term `at` of buffer ab starts at column ab * a_cols + at * Kn / 2,
         // 8 columns per K step
         const uint32_t a_tm0 = tmem_base + 2u * (uint32_t)a.tmem_cols;
         uint32_t a_tmb = a_tm0;  // the current tile's A buffer
-        auto mma_block = [&](uint32_t dtm, uint64_t a0, uint64_t b0, int kb, int at, int brow, uint32_t id,
-                             uint32_t dcol, uint32_t accumulate) {
+        // The descriptors differ in their low words only (start address / 16): those are added up
+        // in 32 bits and joined with the constant high word at each instruction.  Beside warps
+        // that store to shared memory, the 15 MMAs of an N = 35 tile took 2059 cycles issued
+        // with 64-bit descriptor arithmetic and 1447 this way (1008 on the tensor pipe).
+        const uint64_t adesc0 = smem_desc(sbase + offA, W), bdesc0 = smem_desc(sbase, W);
+        const uint32_t a_hi = (uint32_t)(adesc0 >> 32), b_hi = (uint32_t)(bdesc0 >> 32);
+        uint32_t a_lo = (uint32_t)adesc0;
+        const uint32_t b_lo = (uint32_t)bdesc0;
+        auto join = [](uint32_t lo, uint32_t hi) {
+            uint64_t d;
+            asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
+            return d;
+        };
+        auto mma_block = [&](uint32_t dtm, int kb, int at, int brow, uint32_t id, uint32_t accumulate) {
             const int steps = min(KB, Kn - kb * KB) / 16;  // all-zero K steps skipped
-            const uint64_t ad = a0 + ((uint32_t)(at * termA + kb * TE * W) >> 4);
-            const uint64_t bd = b0 + ((uint32_t)(brow * W + kb * bkb) >> 4);
+            const uint32_t ad = a_lo + ((uint32_t)(at * termA + kb * TE * W) >> 4);
+            const uint32_t bd = b_lo + ((uint32_t)(brow * W + kb * bkb) >> 4);
             const uint32_t at_tm = a_tmb + (uint32_t)(at * (Kn / 2) + kb * KB / 2);
 #pragma unroll
             for (int ki = 0; ki < 4; ++ki) {  // at most four K steps of 16 in a K-block of 64
                 if (ki >= steps)
                     break;
                 if (kATmem && a.a_tmem)
-                    tc_mma_ta(dtm + dcol, at_tm + 8u * ki, bd + 2 * ki, id, accumulate);
+                    tc_mma_ta(dtm, at_tm + 8u * ki, join(bd + 2 * ki, b_hi), id, accumulate);
                 else
-                    tc_mma(dtm + dcol, ad + 2 * ki, bd + 2 * ki, id, accumulate);  // +32 bytes per K step
+                    tc_mma(dtm, join(ad + 2 * ki, a_hi), join(bd + 2 * ki, b_hi), id, accumulate);  // +32 bytes per K step
                 accumulate = 1;
             }
         };
         const bool k_outer = NT == 1 || a.stack;
         int k = 0;
-        for (long long t = my_first; t < a.ntiles; t += my_step, ++k) {
-            const int b = k & 1, ab = k % NA;
-            const uint32_t n = (uint32_t)(k >> 1), na = (uint32_t)(k / NA);
+        Ring as;
+        for (long long t = my_first; t < a.ntiles; t += my_step, ++k, as.next(NA)) {
+            const int b = k & 1, ab = as.i;
+            const uint32_t n = (uint32_t)(k >> 1), na = as.ph;
             bool ok = mbar_wait(&acc_empty[b], (n & 1u) ^ 1u);
             const uint32_t dtm = tmem_base + (uint32_t)b * a.tmem_cols;
             a_tmb = a_tm0 + (uint32_t)(ab * a.a_cols);
-            const uint64_t a0 = smem_desc(sbase + offA + (uint32_t)ab * bufA, W);
-            const uint64_t b0 = smem_desc(sbase, W);
+            a_lo = (uint32_t)adesc0 + (((uint32_t)ab * bufA) >> 4);
             const int npass = k_outer ? 1 : 6;
             for (int p = 0; p < npass && ok; ++p) {
                 for (int kb = 0; kb < nkb; ++kb) {
@@ -481,22 +559,23 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
                     if (elect_one()) {
                         const uint32_t acc = kb > 0;  // block 0 of a region's first product overwrites
                         if (NT == 1) {
-                            mma_block(dtm, a0, b0, kb, 0, 0, idesc, 0, acc);
+                            mma_block(dtm, kb, 0, 0, idesc, acc);
                         } else if (a.stack) {
-                            // regions R0 = columns [0, CBp) and R1 = [CBp, 2 CBp), summed by the
+                            // regions R0 = columns [0, CBs) and R1 = [CBs, 2 CBs), summed by the
                             // epilogue: u_hi x [D_hi; D_mid] puts hh in R0 and hm in R1; the
                             // smaller products lh, hl, mm, mh all go to R1, so the large R0 sum
                             // takes one rounding per K step, as a plain FP32 dot product would
-                            mma_block(dtm, a0, b0, kb, 0, 0, idesc2, 0, acc);
-                            mma_block(dtm, a0, b0, kb, 2, 0, idesc, (uint32_t)CBp, 1);
-                            mma_block(dtm, a0, b0, kb, 0, 2 * CBp, idesc, (uint32_t)CBp, 1);
-                            mma_block(dtm, a0, b0, kb, 1, CBp, idesc, (uint32_t)CBp, 1);
-                            mma_block(dtm, a0, b0, kb, 1, 0, idesc, (uint32_t)CBp, 1);
+                            const uint32_t d1 = dtm + (uint32_t)CBs;
+                            mma_block(dtm, kb, 0, 0, idesc2, acc);
+                            mma_block(d1, kb, 2, 0, idesc, 1);
+                            mma_block(d1, kb, 0, 2 * CBs, idesc, 1);
+                            mma_block(d1, kb, 1, CBs, idesc, 1);
+                            mma_block(d1, kb, 1, 0, idesc, 1);
                         } else {
                             // (D term, u term) of pass p: lh, hl, mm, mh, hm, hh
                             const int bt = p == 0 ? 2 : (p == 2 || p == 3) ? 1 : 0;
                             const int at = p == 1 ? 2 : (p == 2 || p == 4) ? 1 : 0;
-                            mma_block(dtm, a0, b0, kb, at, bt * CBp, idesc, 0, p == 0 ? acc : 1u);
+                            mma_block(dtm, kb, at, bt * CBs, idesc, p == 0 ? acc : 1u);
                         }
                         if (p == npass - 1)
                             tc_commit(&a_empty[ab * kTcMaxKB + kb]);
@@ -522,11 +601,11 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
         // the epilogue warps never wait on the bulk-copy engine themselves.
         if (!NODE && a.store_quarters == 4) {
             const int R = a.obufs;
-            int k = 0;
+            Ring os;
             bool ok = true;
-            for (long long t = my_first; t < a.ntiles; t += my_step, ++k) {
-                const int s = k % R;
-                if (!mbar_wait(&slot_full[s], (uint32_t)(k / R) & 1u)) {
+            for (long long t = my_first; t < a.ntiles; t += my_step, os.next(R)) {
+                const int s = os.i;
+                if (!mbar_wait(&slot_full[s], os.ph)) {
                     ok = false;
                     break;
                 }
@@ -567,22 +646,30 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
         // chunks c8_lo + part, c8_lo + part + Hc, ...  The A terms go to shared memory (hardware
         // swizzle) or to tensor memory (tcgen05.st into this warp's lane quarter, warp-uniform
         // loops; rows past the tile and nodes past N are zeros).
-        // Early release (descriptor prefetch_smem = 2): when K is one block and a thread has at
-        // most kMaxEarly chunks, it loads them, splits them into their terms in registers and
-        // hands the u stage back to the producer at once, so the next tile's bulk copy overlaps
-        // this tile's conversion and MMAs, and only the stores of the terms wait for the A
-        // buffer (threads with more chunks take the plain path).
-        // chunks a thread may hold: three (BF16, one term each) or two (three terms each)
-        constexpr int kMaxEarly = NT == 1 ? 3 : 2;
+        // Early release (descriptor prefetch_smem = 2): when no thread has more than kMaxEarly chunks,
+        // each loads all of its own and hands the u stage back to the producer at once, so the next
+        // tile's bulk copy overlaps this tile's conversion and MMAs (else the plain path is taken).
+        constexpr int kMaxEarly = 3;  // chunks (8 values each) a thread may hold
         int k = 0;
         bool ok = true;
         const int nch8 = Kz8 / 8;
-        const int my_chunks = (nkb == 1 && a.early_release) ? (nch8 - part + Hc - 1) / Hc : kMaxEarly + 1;
+        // (one choice for all conversion warps: the plain path deals the chunks out per K-block)
+        const bool early = a.early_release && (nch8 + Hc - 1) / Hc <= kMaxEarly;
+        const int my_chunks = (nch8 - part + Hc - 1) / Hc;
         const uint32_t lane_q = (uint32_t)(32 * (warp & 3)) << 16;
-        for (long long t = my_first; t < a.ntiles && ok; t += my_step, ++k) {
-            const int s = k % S, ab = k % NA;
-            const uint32_t ns = (uint32_t)(k / S), na = (uint32_t)(k / NA);
-            if (!mbar_wait(&u_full[s], ns & 1u)) {
+        // this row's part of swz_off, and the log2 of the chunks in a K-block
+        const uint32_t row_off = (uint32_t)(row * W);
+        const int row_x = (row * W >> 7) & (W / 16 - 1), kb_shift = KB == 64 ? 3 : (KB == 32 ? 2 : 1);
+        // element-major rows of whole 16- or 8-byte pieces are read as such: N = 84 has 4-way bank
+        // conflicts on 4-byte reads (row stride 84) and none on 16-byte reads
+        const std::true_type kStaged{};
+        const std::false_type kGlobal{};
+        const int jvec = NODE ? 1 : (N % 4 == 0 ? 4 : (N % 2 == 0 ? 2 : 1));
+        Ring us, as;
+        for (long long t = my_first; t < a.ntiles && ok; t += my_step, us.next(S), as.next(NA)) {
+            const int s = us.i, ab = as.i;
+            const uint32_t na = as.ph;
+            if (!mbar_wait(&u_full[s], us.ph)) {
                 ok = false;
                 break;
             }
@@ -594,27 +681,41 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
             const bool rowv = row < TEv;
             constexpr int JS = NODE ? TE : 1;
             const float *src_s = NODE ? st + row : st + row * N;
-            const float *src_g = NODE ? a.u + e0 + row : a.u + (e0 + row) * N;
-            const long long jsg = NODE ? E : 1;
             const uint32_t abase = tmem_base + 2u * (uint32_t)a.tmem_cols + (uint32_t)(ab * a.a_cols) + lane_q;
-            // the 8 values of chunk c8 of this thread's row (zeros past the row or past N)
-            auto load_chunk = [&](int c8, float *x) {
-                if (from_stage && c8 * 8 + 8 <= N) {
+            // the 8 values of chunk c8 of this thread's row, zeros past N.  Staged: a row past the
+            // tile's last element reads what the stage holds; its products reach only its own
+            // accumulator lane, which is never stored.
+            auto load_chunk = [&](auto staged, int c8, float *x) {
+                if constexpr (decltype(staged)::value) {
+                    const float *p = src_s + c8 * 8 * JS;
+                    if (c8 * 8 + 8 <= N) {
+                        if (!NODE && jvec == 4) {
+                            const float4 v0 = reinterpret_cast<const float4 *>(p)[0], v1 = reinterpret_cast<const float4 *>(p)[1];
+                            x[0] = v0.x, x[1] = v0.y, x[2] = v0.z, x[3] = v0.w;
+                            x[4] = v1.x, x[5] = v1.y, x[6] = v1.z, x[7] = v1.w;
+                        } else if (!NODE && jvec == 2) {
 #pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        x[q] = rowv ? src_s[(c8 * 8 + q) * JS] : 0.f;
-                } else if (from_stage) {
+                            for (int q = 0; q < 4; ++q) {
+                                const float2 v = reinterpret_cast<const float2 *>(p)[q];
+                                x[2 * q] = v.x, x[2 * q + 1] = v.y;
+                            }
+                        } else {
 #pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        x[q] = (rowv && c8 * 8 + q < N) ? src_s[(c8 * 8 + q) * JS] : 0.f;
+                            for (int q = 0; q < 8; ++q)
+                                x[q] = p[q * JS];
+                        }
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < 8; ++q)
+                            x[q] = c8 * 8 + q < N ? p[q * JS] : 0.f;
+                    }
                 } else {
-                    // unaligned tail tile, read from global memory
+                    // unaligned tile, read from global memory
 #pragma unroll
                     for (int q = 0; q < 8; ++q)
-                        x[q] = (rowv && c8 * 8 + q < N) ? src_g[(long long)(c8 * 8 + q) * jsg] : 0.f;
+                        x[q] = (rowv && c8 * 8 + q < N) ? a.u[NODE ? (c8 * 8 + q) * E + e0 + row : (e0 + row) * N + c8 * 8 + q] : 0.f;
                 }
             };
-            // chunk c8 -> the A terms
             // the NT terms of chunk c8 -> the A buffer
             auto put_terms = [&](int c8, const uint4 *tt4) {
                 if (kATmem && a.a_tmem) {
@@ -622,8 +723,9 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
                     for (int tt = 0; tt < NT; ++tt)
                         tmem_st4(abase + (uint32_t)(tt * (Kn / 2) + c8 * 4), tt4[tt]);
                 } else {
-                    const int kb = (c8 * 8) / KB, ch = ((c8 * 8) % KB) / 8;
-                    const uint32_t off = (uint32_t)kb * TE * W + swz_off(row, ch, W);
+                    // K-block c8 / (KB / 8), swizzled 16-byte chunk of this row (swz_off)
+                    const int kb = c8 >> kb_shift, ch = c8 - (kb << kb_shift);
+                    const uint32_t off = (uint32_t)kb * TE * W + row_off + ((uint32_t)(ch ^ row_x) << 4);
 #pragma unroll
                     for (int tt = 0; tt < NT; ++tt)
                         *reinterpret_cast<uint4 *>(Ab + off + tt * termA) = tt4[tt];
@@ -646,39 +748,61 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
                 if (lane == 0)
                     mbar_arrive(&a_full[ab * kTcMaxKB + kb]);
             };
-            bool released = false;
-            if (from_stage && my_chunks <= kMaxEarly) {
-                // the chunks are split into their terms before the A buffer is free, so that
-                // only the stores of the terms wait for the MMAs of the previous tile
-                uint4 tv[kMaxEarly][3];
-#pragma unroll
-                for (int m = 0; m < kMaxEarly; ++m) {
-                    const int c8 = part + Hc * m;
+            // chunks c8, c8 + Hc, ... below c8_hi, two in flight (uniform across the warp: tcgen05.st
+            // is warp-collective)
+            auto convert = [&](auto staged, int c8, int c8_hi) {
+                for (; c8 < c8_hi; c8 += Hc) {
                     float x[8];
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        x[q] = (m < my_chunks && rowv && c8 * 8 + q < N) ? src_s[(c8 * 8 + q) * JS] : 0.f;
-                    split8<NT>(x, tv[m]);
+                    load_chunk(staged, c8, x);
+                    put(c8, x);
                 }
-                // the loads are complete before the stage is handed back (no load may be
-                // deferred past the arrive to the point where the values are used)
+            };
+            bool released = false;
+            if (from_stage && early) {
+                float xv[kMaxEarly][8];
+                uint32_t all = 0;
+#pragma unroll
+                for (int m = 0; m < kMaxEarly; ++m)
+                    if (m < my_chunks) {
+                        load_chunk(kStaged, part + Hc * m, xv[m]);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q)
+                            all |= __float_as_uint(xv[m][q]);
+                    }
+                // Every load must have returned before the stage is handed back: a fence orders
+                // the instructions, but the arrive overtakes loads that still queue (8-way bank
+                // conflicts at N = 96) and the next bulk copy then overwrites what they read.  The
+                // branch depends on every loaded value, and the arrive on the branch.
+                if (all == 0x7fb5a5a5u)
+                    __nanosleep(0);
                 __threadfence_block();
                 __syncwarp();
                 if (lane == 0)
                     mbar_arrive(&u_empty[s]);  // the stage is free for the next bulk copy
                 released = true;
-                if (!mbar_wait(&a_empty[ab * kTcMaxKB], (na & 1u) ^ 1u)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
+                int kb = 0;
+                auto claim = [&](int q) {  // K-block q of the A buffer is free
+                    const bool got = mbar_wait(&a_empty[ab * kTcMaxKB + q], (na & 1u) ^ 1u);
+                    tc_fence_after();
+                    return got;
+                };
+                ok = claim(0);
 #pragma unroll
                 for (int m = 0; m < kMaxEarly; ++m)
-                    if (m < my_chunks)
-                        put_terms(part + Hc * m, tv[m]);
-                block_done(0);
+                    if (m < my_chunks && ok) {
+                        const int c8 = part + Hc * m;
+                        for (; kb < c8 >> kb_shift && ok; ++kb) {
+                            block_done(kb);
+                            ok = claim(kb + 1);
+                        }
+                        put(c8, xv[m]);
+                    }
+                for (; kb < nkb && ok; ++kb) {
+                    block_done(kb);
+                    if (kb + 1 < nkb)
+                        ok = claim(kb + 1);
+                }
             } else {
-                const int full8 = rowv ? N / 8 : 0;  // chunks with all 8 values inside the row
                 for (int kb = 0; kb < nkb; ++kb) {
                     if (!mbar_wait(&a_empty[ab * kTcMaxKB + kb], (na & 1u) ^ 1u)) {
                         ok = false;
@@ -686,46 +810,10 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
                     }
                     tc_fence_after();
                     const int c8_lo = kb * KB / 8, c8_hi = min(Kz8, (kb + 1) * KB) / 8;
-                    if (kATmem && a.a_tmem) {
-                        // tcgen05.st is warp-collective: every lane runs the same chunks (the
-                        // trip count depends on the warp's share only), rows past the tile are
-                        // zeros by predicated loads
-                        for (int c8 = c8_lo + part; c8 < c8_hi; c8 += Hc) {
-                            float x[8];
-                            load_chunk(c8, x);
-                            put(c8, x);
-                        }
-                    } else if (from_stage) {
-                        // staged tile: compile-time stride along j; two whole chunks in flight, then
-                        // the chunks cut by N or past the tile (zeros) one by one
-                        const int f_hi = min(full8, c8_hi);
-                        int c8 = c8_lo + part;
-                        for (; c8 + Hc < f_hi; c8 += 2 * Hc) {
-                            float x[8], y[8];
-                            const float *p0 = src_s + c8 * 8 * JS, *p1 = src_s + (c8 + Hc) * 8 * JS;
-#pragma unroll
-                            for (int q = 0; q < 8; ++q) {
-                                x[q] = p0[q * JS];
-                                y[q] = p1[q * JS];
-                            }
-                            put(c8, x);
-                            put(c8 + Hc, y);
-                        }
-                        for (; c8 < c8_hi; c8 += Hc) {
-                            float x[8];
-                            const float *p0 = src_s + c8 * 8 * JS;
-#pragma unroll
-                            for (int q = 0; q < 8; ++q)
-                                x[q] = (rowv && c8 * 8 + q < N) ? p0[q * JS] : 0.f;
-                            put(c8, x);
-                        }
-                    } else {
-                        for (int c8 = c8_lo + part; c8 < c8_hi; c8 += Hc) {
-                            float x[8];
-                            load_chunk(c8, x);
-                            put(c8, x);
-                        }
-                    }
+                    if (from_stage)
+                        convert(kStaged, c8_lo + part, c8_hi);
+                    else
+                        convert(kGlobal, c8_lo + part, c8_hi);
                     block_done(kb);
                 }
             }
@@ -758,68 +846,47 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
         const int SQ = NODE ? 4 : a.store_quarters;
         const int NWT = NW * 32;
         const bool stack = NT == 3 && a.stack;
-        // Load, sum and store the chunks of columns [c_begin, c_end) of this warp's lane
-        // quarter; element-major values go to stage + ((operator - f_stage) * TE + row) * N.
+        const std::true_type kStacked{};
+        const std::false_type kPlain{};
+        // Load, sum and store the chunks cc, cc + CW * He, ... below c_end of this warp's lane
+        // quarter.  Element-major values go to `orow`, this thread's row of the staged tile (every
+        // operator, `whole`) or of one operator's slot; node-major ones to column c's output row
+        // at `grow` + row * E.
         // operators packed without padding (Np = N, N not a multiple of the chunk): a chunk of
         // columns c = f N + i may run into the next operator
         const bool packed = Np == N && N % CW != 0;
-        auto drain = [&](int c_begin, int c_end, const uint32_t tbase, float *stage, int f_stage, long long e0,
-                         int TEv) {
+        const bool vec_o = (N & 3) == 0;  // 16-byte aligned staged rows
+        const int step = CW * He;
+        auto drain = [&](auto stacked, int cc, const int c_end, const uint32_t tbase, bool whole, float *orow,
+                         float *grow, bool rowv) {
+            constexpr bool ST = decltype(stacked)::value;
             constexpr int EB = EpiBatch<NT, CW>::value;
-            for (int c0 = c_begin + part * CW; c0 < c_end; c0 += EB * CW * He) {
-                uint32_t r[EB][CW], r2[EB][CW];
+            for (; cc < c_end; cc += EB * step) {
+                uint32_t r[EB][CW], r2[ST ? EB : 1][CW];
 #pragma unroll
-                for (int k4 = 0; k4 < EB; ++k4)
-                    if (c0 + k4 * CW * He < c_end) {
-                        tmem_ld<CW>(tbase + (uint32_t)(c0 + k4 * CW * He), r[k4]);
-                        if (stack)
-                            tmem_ld<CW>(tbase + (uint32_t)(CBp + c0 + k4 * CW * He), r2[k4]);
+                for (int k4 = 0; k4 < EB; ++k4) {
+                    const int ck = cc + k4 * step;
+                    if (ck < c_end) {
+                        tmem_ld<CW>(tbase + (uint32_t)ck, r[k4]);
+                        if (ST)
+                            tmem_ld<CW>(tbase + (uint32_t)(CBs + ck), r2[k4]);
                     }
+                }
                 tmem_wait();
 #pragma unroll
                 for (int k4 = 0; k4 < EB; ++k4) {
-                    const int cc = c0 + k4 * CW * He;
-                    if (cc >= c_end)
+                    const int ck = cc + k4 * step;
+                    if (ck >= c_end)
                         continue;
-                    const int fl = cc / Np, i0 = cc - fl * Np;
-                    const int nv = min(CW, N - i0);  // valid columns of this chunk (>= 1)
-                    if (stack) {
-#pragma unroll
-                        for (int qq = 0; qq < CW; ++qq)
-                            r[k4][qq] = __float_as_uint(__uint_as_float(r[k4][qq]) + __uint_as_float(r2[k4][qq]));
-                    }
-                    if (packed) {
-                        if (NODE) {
-                            if (row < TEv) {
-                                float *o = a.out + ((size_t)f0 * N + cc) * E + e0 + row;  // (f0 + f) N + i = f0 N + c
-#pragma unroll
-                                for (int qq = 0; qq < CW; ++qq) {
-                                    if (cc + qq < c_end)
-                                        *o = __uint_as_float(r[k4][qq]);
-                                    o += E;
-                                }
-                            }
-                        } else {
-                            // (f, row, i) at (f TE + row) N + i: past the operator's last node the
-                            // next operator's row starts (TE - 1) N further on
-                            float *o = stage + ((fl - f_stage) * TE + row) * N + i0;
-                            const int jump = (TE - 1) * N, rest = N - i0;
-                            if (rest >= CW && cc + CW <= c_end) {
-#pragma unroll
-                                for (int qq = 0; qq < CW; ++qq)  // the chunk inside one operator
-                                    o[qq] = __uint_as_float(r[k4][qq]);
-                            } else {
-#pragma unroll
-                                for (int qq = 0; qq < CW; ++qq)
-                                    if (cc + qq < c_end)
-                                        o[qq + (qq >= rest ? jump : 0)] = __uint_as_float(r[k4][qq]);
-                            }
-                        }
-                        continue;
-                    }
+                    const int2 at = chunk_tab[ck / CW];
+                    const int rest = at.y;  // nodes from this chunk's first column on
+                    if (ST)
+                        add_regions<CW>(r[k4], r2[k4]);
                     if (NODE) {
-                        if (row < TEv) {
-                            float *o = a.out + ((size_t)(f0 + fl) * N + i0) * E + e0 + row;
+                        if (rowv) {
+                            float *o = grow + (long long)at.x * E;
+                            // packed columns run on into the next operator's rows
+                            const int nv = packed ? c_end - ck : rest;
 #pragma unroll
                             for (int qq = 0; qq < CW; ++qq) {
                                 if (qq < nv)
@@ -828,22 +895,21 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
                             }
                         }
                     } else {
-                        float *o = stage + ((fl - f_stage) * TE + row) * N + i0;
-                        if ((N & 3) == 0) {
-                            // 16-byte aligned rows: vector stores (nv is a multiple of 4)
-#pragma unroll
-                            for (int h = 0; h < CW / 4; ++h)
-                                if (4 * h < nv)
-                                    *reinterpret_cast<uint4 *>(o + 4 * h) =
-                                        make_uint4(r[k4][4 * h], r[k4][4 * h + 1], r[k4][4 * h + 2], r[k4][4 * h + 3]);
-                        } else if (nv == CW) {
+                        float *o = orow + (whole ? at.x : N - rest);
+                        if (rest >= CW) {
+                            store_chunk<CW>(o, r[k4], vec_o);  // the chunk inside one operator
+                        } else if (packed) {
+                            // past the operator's last node the next operator's row starts
+                            // (TE - 1) N further on
+                            const int jump = (TE - 1) * N;
 #pragma unroll
                             for (int qq = 0; qq < CW; ++qq)
-                                o[qq] = __uint_as_float(r[k4][qq]);
+                                if (ck + qq < c_end)
+                                    o[qq + (qq >= rest ? jump : 0)] = __uint_as_float(r[k4][qq]);
                         } else {
 #pragma unroll
                             for (int qq = 0; qq < CW; ++qq)
-                                if (qq < nv)
+                                if (qq < rest)
                                     o[qq] = __uint_as_float(r[k4][qq]);
                         }
                     }
@@ -853,14 +919,16 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
         // Geometric factors of this thread's element (row) for the current tile: rr[d][f].
         constexpr int FGm = FG > 0 ? FG : 1;
         float rr[FGm][FGm];
-        auto load_r = [&](long long e0, int TEv) {
+        auto load_r = [&](float (&to)[FGm][FGm], long long t) {
+            const long long e0 = t * TE;
+            const bool in = t < a.ntiles && e0 + row < E;
 #pragma unroll
             for (int d = 0; d < FGm; ++d)
 #pragma unroll
                 for (int f = 0; f < FGm; ++f) {
                     const long long e = e0 + row;
-                    rr[d][f] = row >= TEv ? 0.f
-                                          : (NODE ? a.r[((long long)d * FGm + f) * E + e]
+                    to[d][f] = !in ? 0.f
+                                   : (NODE ? a.r[((long long)d * FGm + f) * E + e]
                                                   : a.r[(e * FGm + d) * FGm + f]);
                 }
         };
@@ -875,7 +943,7 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
                     uint32_t r0[CW], r1[CW];
                     tmem_ld<CW>(tbase + (uint32_t)(f * Np + c0), r0);
                     if (stack)
-                        tmem_ld<CW>(tbase + (uint32_t)(CBp + f * Np + c0), r1);
+                        tmem_ld<CW>(tbase + (uint32_t)(CBs + f * Np + c0), r1);
                     tmem_wait();
 #pragma unroll
                     for (int qq = 0; qq < CW; ++qq)
@@ -923,29 +991,35 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
         bool ok = true;
         if (SQ == 4) {
             // ---- node-major, or element-major with whole-tile slots
-            for (long long t = my_first; t < a.ntiles; t += my_step, ++k) {
+            Ring os;
+            for (long long t = my_first; t < a.ntiles; t += my_step, ++k, os.next(R)) {
                 const int b = k & 1;
                 const long long e0 = t * TE;
                 const int TEv = (int)min((long long)TE, E - e0);
+                if (FG > 0)
+                    load_r(rr, t);  // before the wait, which hides the loads
                 const bool got = mbar_wait(&acc_full[b], (uint32_t)((k >> 1) & 1));
-                float *ost = ost0 + (size_t)(k % R) * G * TE * N;
+                float *ost = ost0 + os.i * (G * TE * N);
                 // every warp goes its own way (no named barrier; every wait is bounded)
                 if (!got || *abort_flag) {
                     ok = got;
                     break;
                 }
                 // element-major: the store warp has finished reading this slot
-                if (!NODE && !mbar_wait(&slot_empty[k % R], ((uint32_t)(k / R) & 1u) ^ 1u)) {
+                if (!NODE && !mbar_wait(&slot_empty[os.i], os.ph ^ 1u)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
                 const uint32_t tbase = tmem_base + (uint32_t)b * a.tmem_cols + ((uint32_t)(q * 32) << 16);
                 if (FG > 0) {
-                    load_r(e0, TEv);
                     drain_geo(tbase, ost, e0, TEv);
                 } else {
-                    drain(0, Gb * Np, tbase, ost, 0, e0, TEv);
+                    float *grow = NODE ? a.out + (size_t)f0 * N * E + e0 + row : nullptr;
+                    if (stack)
+                        drain(kStacked, part * CW, Gb * Np, tbase, true, ost + row * N, grow, row < TEv);
+                    else
+                        drain(kPlain, part * CW, Gb * Np, tbase, true, ost + row * N, grow, row < TEv);
                 }
                 release_acc(b);
                 if (!NODE) {
@@ -953,7 +1027,7 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
                     fence_async_smem();
                     __syncwarp();
                     if (lane == 0)
-                        mbar_arrive(&slot_full[k % R]);
+                        mbar_arrive(&slot_full[os.i]);
                 }
             }
         } else {
@@ -971,7 +1045,7 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
                 }
             };
             const int r0 = 32 * SQ * gq;  // first tile row of this store group
-            int ns = 0;                   // slots used by this store group
+            Ring os;                      // slots used by this store group
             for (long long t = my_first; t < a.ntiles; t += my_step, ++k) {
                 const int b = k & 1;
                 const long long e0 = t * TE;
@@ -981,8 +1055,8 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
                 const uint32_t tbase = tmem_base + (uint32_t)b * a.tmem_cols + ((uint32_t)(q * 32) << 16);
                 bool stop = false;
                 for (int g = 0; g < Gb; ++g) {
-                    float *slot = ost0 + (size_t)(ns % R) * TE * N;  // [TE][N], this group's rows r0..
-                    ++ns;
+                    float *slot = ost0 + os.i * (TE * N);  // [TE][N], this group's rows r0..
+                    os.next(R);
                     if (leader)
                         bulk_wait_read(R - 1);  // the store that last read this slot is done reading
                     if (g > 0) {
@@ -995,7 +1069,10 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
                         }
                         tc_fence_after();
                     }
-                    drain(g * Np, (g + 1) * Np, tbase, slot, g, e0, TEv);
+                    if (stack)
+                        drain(kStacked, g * Np + part * CW, (g + 1) * Np, tbase, false, slot + row * N, nullptr, true);
+                    else
+                        drain(kPlain, g * Np + part * CW, (g + 1) * Np, tbase, false, slot + row * N, nullptr, true);
                     if (g == Gb - 1)
                         release_acc(b);
                     fence_async_smem();
