@@ -1251,7 +1251,7 @@ static lc_status resolve(const Kernel &K, long long E, int N, int F, const lc_va
             off += (size_t)q.nkb * (NT * q.CBs + q.CBp - q.CBs) * W;     // B terms
             off += a_tm ? 0 : (size_t)q.abufs * NT * q.nkb * 128 * W;  // A terms
             q.off_stage = (unsigned)off;
-            off += (size_t)q.stages * 128 * N * 4;
+            off += (size_t)q.stages * q.u_ld * N * 4;
             q.off_out = (unsigned)off;
             if (!node)  // staging slots: every operator of the block (4 quarters per store), else one
                 off += (size_t)q.obufs * (q.store_quarters == 4 ? G : 1) * 128 * N * 4;
@@ -1278,6 +1278,9 @@ static lc_status resolve(const Kernel &K, long long E, int N, int F, const lc_va
         // reading A from tensor memory measured slower beside the epilogue's loads); BF16X3
         // takes tensor-memory A where no shared-memory plan fits (N above about 100)
         const bool tm_first = v->a_operand == 2 || (v->a_operand == 0 && NT == 1);
+        // (node-major rows that are not 16-byte aligned need stage rows of 132 values; where that
+        // does not fit, the tiles are read from global memory)
+        for (int shifted = node && E % 4 != 0 ? 1 : 0; shifted >= 0 && !found; --shifted)
         for (int g = g_hi; g >= g_lo && !found; --g)
             for (int pass = 0; pass < 2 && !found; ++pass) {
                 const bool a_tm = tm_first ? pass == 0 : pass == 1;
@@ -1288,6 +1291,8 @@ static lc_status resolve(const Kernel &K, long long E, int N, int F, const lc_va
                 for (int stacked = (a_tm && NT == 3) ? 1 : 0; stacked >= 0 && !found; --stacked)
                     for (int c = 0; c < ncombos && !found; ++c) {
                         TcArgs q = t;
+                        q.u_ld = shifted ? 132 : 128;
+                        q.bulk_u = shifted ? 2 : (!node || E % 4 == 0);
                         q.obufs = node ? 1 : combos[c][0];
                         q.abufs = combos[c][1];
                         if (!node && v->out_buffers && q.obufs != v->out_buffers)
@@ -1306,7 +1311,6 @@ static lc_status resolve(const Kernel &K, long long E, int N, int F, const lc_va
         // element-major whole-tile slots: the store warp issues the bulk stores and waits for
         // their reads, so the epilogue warps go on to the next tile at once
         t.store_warp = !node && t.store_quarters == 4;
-        t.bulk_u = node ? (E % 4 == 0) : 1;
         t.bulk_store = !node && ((E * (long long)N) % 4 == 0);
         long long work = t.ntiles * t.nblocks;
         long long grid = std::min<long long>(work, (long long)sms);
@@ -1988,6 +1992,11 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
                     take(2, 2, stg, 1, 32, 1, 0, all_ops);
             for (int stg : {3, 2, 1})
                 take(2, 1, stg, 64, N > 80 ? 32 : 128, 2, 1, stacked);
+        } else if (!x3 && geo) {
+            // (the geometric-factor epilogue does more per value: four threads a row)
+            for (int stg : {2, 3, 1})
+                for (int kbw : {64, 1})
+                    take(4, 1, stg, kbw, 0, 0, 0, any);
         } else if (!x3 && !node) {
             // BF16: many warps up to N = 48 (N = 35, F = 3, E = 2^20: 99 us), fewer above (N = 120,
             // F = 3, E = 2^18: 92 against 105)

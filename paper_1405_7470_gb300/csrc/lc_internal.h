@@ -157,7 +157,9 @@ struct TcArgs {
     int store_quarters;  // element-major: TMEM lane quarters (32 rows each) per bulk store: 1, 2 or 4
     int store_warp;      // 1: whole-tile element-major slots are written out by the CTA's store warp
     long long ntiles;
-    int bulk_u, bulk_store;
+    int bulk_u;     // u tiles by the bulk engine: 1, or 2 = node-major rows not 16-byte aligned (E % 4 != 0)
+    int u_ld;       // node-major: values between staged rows (128, or 132 with bulk_u 2)
+    int bulk_store;
     unsigned int *err;
     unsigned int off_stage, off_out, off_bar, smem_bytes;
 };

@@ -452,11 +452,23 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_holder, 0);
 
+    // Node-major rows of u (E values) start on 16-byte boundaries only if E % 4 == 0.  Otherwise
+    // (a.bulk_u == 2) row j's copy starts up to 3 values early, at the boundary before it, into a
+    // stage row of 132 values, and the readers skip row_shift(j) values; the last tiles, whose
+    // copies could run past the array, are read from global memory.  (N = 20, F = 2, odd E: every
+    // tile went through 4-byte global loads by the conversion warps.)
+    auto row_shift = [&](int j) { return (int)((unsigned)(j & 3) * (unsigned)(E & 3) & 3u); };
     // bulk-copy bytes of u tile t (0: not fetchable by the bulk engine, read from global)
     auto tile_bulk_bytes = [&](long long t) -> uint32_t {
-        const int TEv = (int)min((long long)TE, E - t * TE);
+        const long long left = E - t * TE;
+        const int TEv = (int)min((long long)TE, left);
         if (!a.bulk_u)
             return 0;
+        if (NODE && a.bulk_u == 2) {
+            // rows without a shift: every fourth (odd E) or second
+            const int n0 = (E & 1) ? (N + 3) / 4 : (N + 1) / 2;
+            return left >= TE + 4 ? (uint32_t)(N * (TE + 4) - 4 * n0) * 4u : 0u;
+        }
         const uint32_t bytes = (uint32_t)TEv * N * 4u;
         return (bytes & 15u) ? 0u : bytes;
     };
@@ -482,10 +494,18 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
                 mbar_arrive_expect_tx(&u_full[s], bytes);
             __syncwarp();
             if (bytes) {
-                float *dst = stage + (size_t)s * TE * N;
+                float *dst = stage + s * (a.u_ld * N);
                 if (NODE) {
-                    for (int j = lane; j < N; j += 32)
-                        bulk_g2s(dst + (size_t)j * TE, a.u + (size_t)j * E + e0, (uint32_t)TEv * 4u, &u_full[s]);
+                    if (a.bulk_u == 2) {
+                        for (int j = lane; j < N; j += 32) {
+                            const int sh = row_shift(j);
+                            bulk_g2s(dst + j * (TE + 4), a.u + (size_t)j * E + e0 - sh, sh ? (TE + 4) * 4u : TE * 4u,
+                                     &u_full[s]);
+                        }
+                    } else {
+                        for (int j = lane; j < N; j += 32)
+                            bulk_g2s(dst + j * TE, a.u + (size_t)j * E + e0, (uint32_t)TEv * 4u, &u_full[s]);
+                    }
                 } else if (lane == 0) {
                     bulk_g2s(dst, a.u + e0 * N, bytes, &u_full[s]);
                 }
@@ -662,8 +682,10 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
         const int row_x = (row * W >> 7) & (W / 16 - 1), kb_shift = KB == 64 ? 3 : (KB == 32 ? 2 : 1);
         // element-major rows of whole 16- or 8-byte pieces are read as such: N = 84 has 4-way bank
         // conflicts on 4-byte reads (row stride 84) and none on 16-byte reads
-        const std::true_type kStaged{};
-        const std::false_type kGlobal{};
+        const std::integral_constant<int, 0> kGlobal{};
+        const std::integral_constant<int, 1> kStaged{};
+        const std::integral_constant<int, 2> kShifted{};  // node-major, E % 4 != 0
+        const int shift[4] = {0, row_shift(1), row_shift(2), row_shift(3)};
         const int jvec = NODE ? 1 : (N % 4 == 0 ? 4 : (N % 2 == 0 ? 2 : 1));
         Ring us, as;
         for (long long t = my_first; t < a.ntiles && ok; t += my_step, us.next(S), as.next(NA)) {
@@ -676,7 +698,7 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
             const long long e0 = t * TE;
             const int TEv = (int)min((long long)TE, E - e0);
             const bool from_stage = tile_bulk_bytes(t) != 0;
-            const float *st = stage + (size_t)s * TE * N;
+            const float *st = stage + s * (a.u_ld * N);
             unsigned char *Ab = smem + offA + (size_t)ab * bufA;
             const bool rowv = row < TEv;
             constexpr int JS = NODE ? TE : 1;
@@ -686,7 +708,12 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
             // tile's last element reads what the stage holds; its products reach only its own
             // accumulator lane, which is never stored.
             auto load_chunk = [&](auto staged, int c8, float *x) {
-                if constexpr (decltype(staged)::value) {
+                if constexpr (NODE && decltype(staged)::value == 2) {
+                    const float *p = src_s + c8 * 8 * (TE + 4);  // (chunks start at a multiple of 4 rows)
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)
+                        x[q] = c8 * 8 + q < N ? p[q * (TE + 4) + shift[q & 3]] : 0.f;
+                } else if constexpr (decltype(staged)::value == 1) {
                     const float *p = src_s + c8 * 8 * JS;
                     if (c8 * 8 + 8 <= N) {
                         if (!NODE && jvec == 4) {
@@ -758,7 +785,7 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
                 }
             };
             bool released = false;
-            if (from_stage && early) {
+            if (from_stage && early && !(NODE && a.bulk_u == 2)) {
                 float xv[kMaxEarly][8];
                 uint32_t all = 0;
 #pragma unroll
@@ -810,7 +837,9 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
                     }
                     tc_fence_after();
                     const int c8_lo = kb * KB / 8, c8_hi = min(Kz8, (kb + 1) * KB) / 8;
-                    if (from_stage)
+                    if (NODE && from_stage && a.bulk_u == 2)
+                        convert(kShifted, c8_lo + part, c8_hi);
+                    else if (from_stage)
                         convert(kStaged, c8_lo + part, c8_hi);
                     else
                         convert(kGlobal, c8_lo + part, c8_hi);

@@ -68,3 +68,20 @@ def test_early_release_with_queued_stage_reads(lc, prec, N, F):
         if lc.variant_validate(kernel, E, N, F, v) != 0:
             continue
         assert np.array_equal(run(lc, kernel, v, D, u, "elem"), want), (stages, kbw, aop)
+
+
+# node-major rows that start off the 16-byte boundary by each amount, tiles before and at the
+# point where the last tile's copies would run past the array, N off every chunk size
+@pytest.mark.parametrize("prec", ["bf16", "bf16x3"])
+@pytest.mark.parametrize("E", [128 * 3 + 1, 128 * 3 + 2, 128 * 3 + 3, 128 * 3 + 5, 128 * 3 + 7, 30001, 30002, 131, 130])
+def test_node_major_unaligned_rows(lc, prec, E):
+    kernel = lc.Kernel()
+    for N, F in ((20, 2), (35, 3), (9, 1)):
+        D, u = synth.integer_operands(E, N, F, seed=E + N)
+        uu = synth.to_node_major(u)
+        want = oracle.contract(D, uu, "node")
+        for unroll, prefetch, stages in ((1, 1, 3), (3, 2, 1)):
+            v = lc.Variant(engine="tcgen05", layout="node", precision=prec, tile_e=128, elems_per_thread=64, split_i=0,
+                           unroll=unroll, prefetch_smem=prefetch, stages=stages, store_rows=0, max_ctas=40)
+            assert lc.variant_validate(kernel, E, N, F, v) == 0
+            assert np.array_equal(run(lc, kernel, v, D, uu, "node"), want), (N, unroll)
