@@ -125,7 +125,9 @@ struct lc_variant {
                                  operands, 16, 32 or 64 (1 = widest dividing N rounded to 16) */
     int32_t split_i;          /* ilp tag on i: output columns per thread (SIMT register block);
                                  tensor-core engine: operators per CTA column block (0 = most) */
-    int32_t unroll;           /* unr tag on the j reduction: 1, 2, 4 or 8; tensor-core engine:
+    int32_t unroll;           /* unr tag on the j reduction: 1, 2, 4 or 8 (8 with prefetch_smem 1,
+                                 FP32, N = 13 to 40: j unrolled wholly, the rows of u in
+                                 registers; the other tile fields are then unused); tensor-core engine:
                                  epilogue threads per tile row, 1 to 4 (conversion threads per
                                  row: 1; 2 to 4, growing with N; 3; 2) */
     int32_t prefetch_smem;    /* add_prefetch of the u tile into shared memory by TMA (1) or
@@ -167,8 +169,8 @@ struct lc_variant {
 
 /*
  * A reasonable descriptor for (E, N, F, layout, precision): fills *v.  The choices follow
- * the autotuner's measurements on this GPU: FP32 on the warp engine up to N = 12, SIMT
- * tiles below N = 64, the K-split engine from N = 64; BF16 and BF16X3 on the tensor cores
+ * the autotuner's measurements on this GPU: FP32 on the warp engine up to N = 12, the SIMT
+ * engine below N = 64 (whole rows of u in registers up to N = 40, tiles above), the K-split engine from N = 64; BF16 and BF16X3 on the tensor cores
  * (BF16X3 with the A terms in shared memory or, where that is faster, in tensor memory, up
  * to N = 128), and where no tensor-core plan exists the FP32 kernels, whose error is below both
  * reduced-precision bounds; FP64 SIMT tiles.  No GPU work is done.

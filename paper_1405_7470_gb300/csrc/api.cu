@@ -1142,6 +1142,30 @@ static lc_status resolve(const Kernel &K, long long E, int N, int F, const lc_va
         if (!cap_grid(grid, g.nchunks, v->max_ctas))
             return LC_ERR_INVALID_VARIANT;
         g.grid = (int)grid;
+        // The j loop wholly unrolled (unroll 8) over a staged u: from N = 13 (smaller N has the warp
+        // engine) to 40 (two rows of u and the sums fill 128 registers a thread) the row kernel
+        // runs it, one CTA per SM; E = 2^21, N = 35, F = 3: see simt_row.cu.  Fewer than four
+        // warps (large F, element-major) would leave the FMA pipes waiting.
+        g.row = 0;
+        if (v->precision == LC_PREC_FP32 && v->prefetch_smem && v->unroll == 8 && N >= 13 && N <= 40) {
+            const RowPlan rp = row_plan(E, N, F, node, sms, smem_cap);
+            if (rp.warps >= 4) {
+                g.row = rp.ept;
+                g.parts = rp.parts;
+                g.stages = rp.buffers;
+                g.G = F;
+                g.isplit = 0;
+                g.nchunks = 1;
+                g.TE = 32 * rp.ept;
+                g.ntiles = (E + g.TE - 1) / g.TE;
+                g.threads = 32 * rp.warps;
+                g.smem = rp.smem;
+                grid = std::min<long long>(std::max<long long>(g.ntiles * rp.parts, 1), sms);
+                if (!cap_grid(grid, 1, v->max_ctas))
+                    return LC_ERR_INVALID_VARIANT;
+                g.grid = (int)grid;
+            }
+        }
         return LC_OK;
     }
     if (v->engine == LC_ENGINE_TCGEN05) {
@@ -1891,34 +1915,26 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
                 return LC_OK;
             }
         }
-        // SIMT tiles, two CTAs per SM, the u tile staged by bulk copies two tiles ahead; the
-        // fastest measured per layout and node count (autotuner, N = 20 .. 84, F = 2 .. 4):
-        // element-major 4 x 8 register blocks with j unrolled 4 times, 64-element tiles up to
-        // N = 40 and 32 above (N = 56: 0.58 ms against 1.00 ms for 128-element tiles of 8 x 8
-        // blocks); node-major without unrolling (N = 56: 0.57 against 0.77 ms unrolled)
+        // SIMT.  N <= 40: the row kernel (unroll 8: the whole rows of u in registers); E = 2^21,
+        // F = 3: N = 35 494 -> 351 us element-major, 486 -> 356 node-major; N = 20 280 -> 121 and
+        // 228 -> 142; E = 4099, N = 35: 14.7 -> 10.6 and 21 -> 11.  Above: tiles, two CTAs per SM, the
+        // u tile staged by bulk copies two tiles ahead; element-major 4 x 8 register blocks with
+        // j unrolled 4 times, 32-element tiles (N = 56: 0.58 ms against 1.00 ms for 128-element
+        // tiles of 8 x 8 blocks); node-major without unrolling (N = 56: 0.57 against 0.77 ms unrolled)
         d.engine = LC_ENGINE_SIMT;
         d.ctas_per_sm = 2;
         d.prefetch_smem = 1;
         d.stages = 2;
-        if (layout == LC_LAYOUT_ELEM_MAJOR) {
-            d.elems_per_thread = 4;
-            d.split_i = 8;
-            d.tile_e = N <= 40 ? 64 : 32;
+        d.elems_per_thread = 4;
+        d.split_i = 8;
+        if (N <= 40) {
+            d.tile_e = 64;
+            d.unroll = 8;
+        } else if (layout == LC_LAYOUT_ELEM_MAJOR) {
+            d.tile_e = 32;
             d.unroll = 4;
-        } else if (N <= 24) {
-            d.elems_per_thread = 8;
-            d.split_i = 4;
-            d.tile_e = 128;
-            d.unroll = 4;
-        } else if (N <= 40) {
-            d.elems_per_thread = 8;
-            d.split_i = 8;
-            d.tile_e = 128;
-            d.unroll = 1;
         } else {
-            d.elems_per_thread = 4;
-            d.split_i = 8;
-            d.tile_e = N <= 72 ? 64 : 32;
+            d.tile_e = 64;
             d.unroll = 1;
         }
     } else {
@@ -2108,6 +2124,10 @@ lc_status lc_contract(const lc_kernel *kh, const lc_variant *v, const void *D, c
         a.tail_free = r.tail_free;
         a.err = error_word();
         const bool node = r.layout == LC_LAYOUT_NODE_MAJOR;
+        if (r.g.row) {
+            a.nchunks = r.g.parts;
+            return row_launch(a, r.layout, r.g.row, r.g.grid, r.g.threads, r.g.smem, s);
+        }
         if (r.precision == LC_PREC_FP32)
             return node ? simt_launch_f32_node(a, r.g, r.unroll, r.prefetch, s)
                         : simt_launch_f32_elem(a, r.g, r.unroll, r.prefetch, s);

@@ -73,6 +73,8 @@ struct SimtGeom {
     size_t smem;   // dynamic shared memory bytes
     long long ntiles;
     int grid;
+    int row;       // > 0: the row kernel (simt_row.cu), this many whole u rows in a thread's registers
+    int parts;     // row kernel: units per element chunk
 };
 
 struct SimtArgs {
@@ -238,6 +240,14 @@ lc_status simt_launch_f64_elem(const SimtArgs &a, const SimtGeom &g, int unroll,
                                cudaStream_t s);
 lc_status simt_launch_f64_node(const SimtArgs &a, const SimtGeom &g, int unroll, int prefetch,
                                cudaStream_t s);
+// Row kernel (simt_row.cu).
+struct RowPlan {
+    int ept, warps, buffers;  // elements a thread (a warp's chunk is 32 of them), warps a CTA, buffers a warp
+    int parts;                // units per chunk: 1, or F (one operator each)
+    size_t smem;
+};
+RowPlan row_plan(long long E, int N, int F, bool node, int sms, size_t smem_cap);
+lc_status row_launch(const SimtArgs &a, int layout, int ept, int grid, int threads, size_t smem, cudaStream_t s);
 lc_status warp_launch(const WarpArgs &a, int layout, int fp64, int grid, int threads, cudaStream_t s);
 
 }  // namespace lc

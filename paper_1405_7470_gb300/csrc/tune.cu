@@ -38,6 +38,19 @@ static std::vector<lc_variant> candidates(int N, int F, int layout, int precisio
                         v.ctas_per_sm = 2;
                         out.push_back(v);
                     }
+        if (precision == LC_PREC_FP32 && N >= 13 && N <= 40) {
+            // the whole rows of u in registers
+            lc_variant v = b;
+            v.engine = LC_ENGINE_SIMT;
+            v.elems_per_thread = V;
+            v.split_i = 2 * V;
+            v.tile_e = 64;
+            v.unroll = 8;
+            v.prefetch_smem = 1;
+            v.stages = 2;
+            v.ctas_per_sm = 2;
+            out.push_back(v);
+        }
         if (precision == LC_PREC_FP32) {
             // K-split: tile 64 or 128 elements, j chunks of 8 or 16, one or two u buffers
             for (int bm : {64, 128})
