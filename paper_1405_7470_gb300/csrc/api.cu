@@ -1837,8 +1837,9 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
     if (kh->k.kind == KIND_LIFT) {
         if (precision != LC_PREC_FP32 || layout != LC_LAYOUT_ELEM_MAJOR)
             return LC_ERR_UNSUPPORTED;
-        // one staging buffer, three CTAs per SM (E = 2^21, degree 4: 0.60 ms, against 0.72 ms
-        // with two buffers, where only two CTAs fit)
+        // one staging buffer and tiles of 64: what the row kernel runs; the tiled kernel (more than 64
+        // face nodes) with three CTAs per SM (E = 2^21, degree 4: 0.60 ms, against 0.72 ms with two
+        // buffers, where only two CTAs fit)
         d.engine = LC_ENGINE_SIMT;
         d.precision = LC_PREC_FP32;
         d.tile_e = 64;

@@ -199,9 +199,20 @@ struct LiftArgs {
                            // -1: every operand read from global memory
     int nbuf;              // staging buffers (1 or 2)
     int te;                // elements per tile (64 or 128)
+    int bulk_store;        // row kernel: out is 16-byte aligned
+    int warps;             // row kernel: warps with a chunk of elements each
+    int stage_s;           // row kernel: the scales come with the vmapP rows (else from global memory)
     unsigned int *err;     // device error word: bit 1 set on an index out of range
 };
 lc_status lift_launch(const LiftArgs &a, int grid, cudaStream_t s);
+// Row kernel (lift_row.cu): warps a CTA, halo rows, shared memory, CTA tiles (0 warps: not for this shape)
+struct LiftRowPlan {
+    int ept, warps, halo, stage_s;
+    size_t smem;
+    long long tiles;
+};
+LiftRowPlan lift_row_plan(long long E, int N, int M, int Nf, int sms, size_t smem_cap);
+lc_status lift_row_launch(const LiftArgs &a, int ept, int grid, size_t smem, cudaStream_t s);
 size_t lift_smem_bytes(int N, int M, int Nf, int halo, int nbuf, int te);
 int lift_threads(int N, int te);
 

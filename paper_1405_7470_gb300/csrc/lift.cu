@@ -5,7 +5,8 @@
 // the jumps between each face node's interior trace and the exterior trace gathered through
 // the face-node map vmapP, scaled per face and lifted to the volume nodes.  FP32 throughout
 // (the contraction has K = Nf * Nfp and about 5 flops per byte moved: the FMA pipes are not
-// the limit, so the tensor cores would buy nothing here).
+// the limit, so the tensor cores would buy nothing here).  Up to four faces and 64 face nodes the
+// row kernel (lift_row.cu) runs it; this file holds the entry point and the tiled kernel for the rest.
 //
 // One CTA walks element tiles of TE elements (persistent, grid-stride):
 //   stage    (add_prefetch, descriptor prefetch_smem = 1) the bulk-copy engine fetches, one
@@ -393,7 +394,23 @@ lc_status lc_lift(const lc_kernel *kh, const lc_variant *v, const float *L, cons
     a.halo = halo;
     a.nbuf = nbuf;
     a.te = te;
+    a.bulk_store = ((uintptr_t)out & 15u) == 0;
     a.err = error_word();
+    // The row kernel where its operands can be staged and it holds a row's fluxes (up to four faces and
+    // 64 face nodes); E = 2^21, degree 4: 325 us against 605.  Beyond that (degree 5: M = 84), with two
+    // staging buffers or tiles of 128, the tiled kernel.
+    if (halo >= 0 && nbuf == 1 && te == 64) {
+        const LiftRowPlan p = lift_row_plan(E, N, a.M, Nf, sms, smem_optin_limit());
+        if (p.warps > 0) {
+            a.halo = p.halo;
+            a.stage_s = p.stage_s;
+            a.warps = p.warps;
+            long long grid = std::min<long long>(p.tiles, sms);
+            if (v->max_ctas > 0)
+                grid = std::min<long long>(grid, v->max_ctas);
+            return lift_row_launch(a, p.ept, (int)grid, p.smem, (cudaStream_t)stream);
+        }
+    }
     const long long ntiles = (E + te - 1) / te;
     long long grid = std::min<long long>(ntiles, (long long)(v->ctas_per_sm ? v->ctas_per_sm : 4) * sms);
     if (v->max_ctas > 0)

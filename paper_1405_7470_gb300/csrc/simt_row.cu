@@ -33,49 +33,12 @@
 #include <algorithm>
 
 #include "lc_internal.h"
-#include "tma.cuh"
+#include "row.cuh"
 
 namespace lc {
 
-__host__ __device__ inline int row_np(int N) { return (N + 3) & ~3; }
 // operators: [F N + 3][NP] floats (the column loop reads up to three rows past the last)
 __host__ __device__ inline size_t row_d_bytes(int N, int F) { return sizeof(float) * (size_t)(F * N + 3) * row_np(N); }
-
-// D^T operands of columns c0 .. c0 + 3 against the rows in ur: r[x][m] = out value of element x
-template <int NP, int EPT>
-__device__ __forceinline__ void row_columns(const float *Ds, const uint64_t (&ur)[EPT][NP / 2], float (&r)[EPT][4])
-{
-    uint64_t acc[EPT][4];
-#pragma unroll
-    for (int x = 0; x < EPT; ++x)
-#pragma unroll
-        for (int m = 0; m < 4; ++m)
-            acc[x][m] = 0;
-#pragma unroll
-    for (int q = 0; q < NP / 4; ++q) {
-        ulonglong2 d[4];
-#pragma unroll
-        for (int m = 0; m < 4; ++m)
-            d[m] = *reinterpret_cast<const ulonglong2 *>(Ds + m * NP + 4 * q);
-#pragma unroll
-        for (int m = 0; m < 4; ++m)
-#pragma unroll
-            for (int x = 0; x < EPT; ++x)
-                acc[x][m] = fma_f32x2(ur[x][2 * q], d[m].x, acc[x][m]);
-#pragma unroll
-        for (int m = 0; m < 4; ++m)
-#pragma unroll
-            for (int x = 0; x < EPT; ++x)
-                acc[x][m] = fma_f32x2(ur[x][2 * q + 1], d[m].y, acc[x][m]);
-    }
-#pragma unroll
-    for (int x = 0; x < EPT; ++x)
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const float2 v = unpack_f32x2(acc[x][m]);
-            r[x][m] = v.x + v.y;
-        }
-}
 
 template <int NP, int LAYOUT, int EPT>
 __global__ void __launch_bounds__(EPT == 4 ? 256 : 512, 1) row_contract_kernel(SimtArgs a)
