@@ -1872,11 +1872,23 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
     d.prefetch_smem = 1;
     d.ctas_per_sm = 0;
     if (precision == LC_PREC_FP64) {
+        // The FP64 pipes bound it; what the descriptor decides is how evenly the SMs and their four
+        // schedulers get the work.  Blocks of 2 x 2 in tiles of 32: four times the threads of 4 x 4 in
+        // tiles of 64, and half-empty warps weigh less.  N = 20, F = 1: E = 4096 19.1 -> 9.9 us,
+        // 30000 41.4 -> 29.4, 200000 171 -> 140; N = 48 957 -> 769 and N = 64 1586 -> 1357 at
+        // E = 200000; N = 32 350 -> 348.  Up to N = 12 a batch that fills the SMs is bound by loads
+        // instead: blocks of 4 x 2 in tiles of 64 (N = 10, F = 3, E = 200000 113 us, 2 x 2 128; N = 6,
+        // F = 1 23.3, 2 x 2 27.1, 4 x 4 25.4).
+        const bool wide = N <= 12 && E >= 64 * 152;
         d.engine = LC_ENGINE_SIMT;
-        d.elems_per_thread = 4;
-        d.split_i = 4;
-        d.tile_e = 64;
+        d.elems_per_thread = wide ? 4 : 2;
+        d.split_i = 2;
+        d.tile_e = wide ? 64 : 32;
         d.stages = 2;
+        if (lc_variant_validate(kh, E, N, F, &d) != LC_OK) {  // (operators that fit only the larger blocks)
+            d.elems_per_thread = d.split_i = 4;
+            d.tile_e = 64;
+        }
     } else if (precision == LC_PREC_FP32) {
         if (N >= 64) {
             // large N: the K-split kernel (D^T streamed in chunks of 16 j) against the SIMT
