@@ -338,17 +338,22 @@ __global__ void __launch_bounds__(KsShape<BM, BK, BN>::TH, BM == 128 ? 2 : 3)
     cp_async_wait_all();  // no copy outlives the CTA
 }
 
-// Column block width: the one of the compiled widths that covers C columns with the fewest
-// padded ones (the widest of equals: fewer passes over the u tile in shared memory).
+// Column block width: the one of the compiled widths that covers C columns soonest.
 int ks_block_cols(int C, int bm)
 {
     if (bm != 128)
         return 128;
-    int best = 128;
-    for (int bn : {112, 96, 80, 64})
-        if ((C + bn - 1) / bn * bn < (C + best - 1) / best * best)
-            best = bn;
-    return best;
+    // Time per padded column, in hundredths of a block of 128's (measured, N = 64 to 95: 160 us a unit
+    // of work, 174, 188, 211, ...): a smaller block has fewer warps to hide latency with, and 80 and 112
+    // do not deal them evenly to the four schedulers.  N = 75, F = 3, E = 177780: 255 us with 3 x 80
+    // columns, 198 with 2 x 128; N = 73, F = 4, E = 140742: 261 with 4 x 80, 229 with 3 x 112.
+    const int width[] = {128, 112, 96, 80, 64}, weight[] = {100, 108, 118, 132, 145};
+    int best = 0;
+    auto cost = [&](int q) { return (C + width[q] - 1) / width[q] * width[q] * weight[q]; };
+    for (int q = 1; q < 5; ++q)
+        if (cost(q) < cost(best))
+            best = q;
+    return width[best];
 }
 
 int ks_threads(int bm, int bn) { return (bm / 8) * (bn / 8); }
