@@ -1885,12 +1885,12 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
         d.split_i = 2;
         d.tile_e = wide ? 64 : 32;
         d.stages = 2;
-        if (lc_variant_validate(kh, E, N, F, &d) != LC_OK) {  // (operators that fit only the larger blocks)
-            d.elems_per_thread = d.split_i = 4;
-            d.tile_e = 64;
-        }
     } else if (precision == LC_PREC_FP32) {
-        if (N >= 64) {
+        // Just above 64 two operators' D^T still fit beside two CTAs of the SIMT kernel, and their columns
+        // pad badly (N = 66, F = 2 403 against 534 us, N = 77, F = 2 429 against 477; N = 66, F = 3 407
+        // against 447; at N = 70, F = 3 and N = 66, F = 4 the K-split kernel is ahead).
+        const bool tiles = N > 64 && N < 80 && (F == 2 || (N < 70 && F < 4));
+        if (N >= 64 && !tiles) {
             // large N: the K-split kernel (D^T streamed in chunks of 16 j) against the SIMT
             // kernel holding all of D^T: N = 64, F = 3, E = 2^19 392 against 476 us element-major,
             // 318 against 345 node-major; N = 84, F = 4, E = 2^20 1565 against 1746 and 1342
@@ -1979,6 +1979,21 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
                 st = rs;
         };
         auto any = [](const TcArgs &) { return true; };
+        // a plan with three stages that gives up neither an operator of the block nor an A buffer
+        // against two stages
+        auto no_less = [&](int unroll, int aop, bool buffers) {
+            lc_variant c = d;
+            c.unroll = unroll;
+            c.prefetch_smem = 1;
+            c.stages = 2;
+            c.elems_per_thread = 64;
+            c.store_rows = 0;
+            c.a_operand = aop;
+            c.split_i = 0;
+            const bool fits = resolve(kh->k, E, N, F, &c, r, false) == LC_OK;
+            const int g = fits ? r.tc.G : 0, ab = fits && buffers ? r.tc.abufs : 0;
+            return [g, ab](const TcArgs &t) { return t.G >= g && t.abufs >= ab; };
+        };
         auto roomy = [](const TcArgs &t) { return t.abufs == 2 && t.obufs >= 2; };
         auto all_ops = [F](const TcArgs &t) { return t.G == F; };
         // (three terms with A in tensor memory: only with the large products kept apart, whose
@@ -1990,7 +2005,11 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
             // few warps (one thread a row and role: 352 threads) and deep staging: N = 35, F = 3,
             // E = 2^20 102 us against 114 with 608 threads and two stages; geometric factors
             // need more epilogue threads (139 against 158 us)
-            const int u = geo ? 3 : (N > 48 && N <= 64 ? 2 : 1);
+            const int u = geo ? 3 : ((N > 48 && N <= 64) || N > 96 ? 2 : 1);
+            if (N > 48 && N <= 64)  // (F = 4: three stages cost an A buffer, N = 64 137 us against 110)
+                take(u, 1, 3, 64, 0, 1, 0, no_less(u, 1, true));
+            if (N > 48 && N <= 64)
+                take(u, 1, 2, 64, 0, 1, 0, any);
             for (int stg : {3, 2, 1})
                 for (int kbw : {64, 1})
                     take(u, 1, stg, kbw, 0, 1, 0, any);
@@ -2027,19 +2046,45 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
                 for (int kbw : {64, 1})
                     take(4, 1, stg, kbw, 0, 0, 0, any);
         } else if (!x3 && !node) {
-            // BF16: many warps up to N = 48 (N = 35, F = 3, E = 2^20: 99 us), fewer above (N = 120,
-            // F = 3, E = 2^18: 92 against 105)
+            // BF16: many warps up to N = 48, fewer above.  Three stages where two A buffers and two
+            // slots fit beside them (N = 20, F = 1 229 -> 207 us, N = 50, F = 1 143 -> 128), and between
+            // N = 64 and 96 for several operators (N = 84, F = 3 153 -> 132, N = 70, F = 4 201 -> 144;
+            // for one 128 against 142); narrow K-blocks where only they leave room for both (N = 35,
+            // F = 4 140 -> 132)
             const int u = N <= 48 ? 3 : 2;
+            if (N <= 64) {
+                take(u, 1, 3, 64, 0, 0, 0, roomy);
+                take(u, 1, 2, 64, 0, 0, 0, roomy);
+                if (N <= 48)
+                    take(u, 1, 2, 1, 0, 0, 0, roomy);
+            }
+            if (N > 64 && N < 96 && F > 1)
+                take(u, 1, 3, 64, 0, 0, 0, no_less(u, 0, false));
             for (int stg : {2, 3, 1})
                 for (int kbw : {64, 1})
-                    take(u, 1, stg, N > 96 ? 65 - kbw : kbw, 0, 0, 0, any);
-        } else if (!x3) {
-            // BF16, node-major: N = 35, F = 3, E = 2^20 99 us (111 with two stages); N = 84, F = 4,
-            // E = 2^19 168 (177)
-            const int u = N <= 64 ? 3 : 1;
-            for (int stg : {3, 2, 1})
-                for (int kbw : {64, 1})
                     take(u, 1, stg, kbw, 0, 0, 0, any);
+        } else if (!x3) {
+            // BF16, node-major.  Up to N = 64: three stages, but with many columns two stages and
+            // more threads a row (N = 64, F = 3 147 -> 136 us, N = 56, F = 4 174 -> 159; N = 44, F = 3
+            // 139 against 143).  Up to N = 96: few warps, three stages unless they cost an A
+            // buffer or an operator of the block (N = 77, F = 3 181 against 143 with two).  Above: two stages, two threads
+            // (N = 112, F = 4 165 against 280 with one and three stages).
+            if (N <= 64 && F * N >= 140)
+                for (int kbw : {64, 1})
+                    take(4, 1, 2, kbw, 0, 0, 0, any);
+            if (N <= 64)
+                for (int stg : {3, 2, 1})
+                    for (int kbw : {64, 1})
+                        take(3, 1, stg, kbw, 0, 0, 0, any);
+            if (N <= 96) {
+                take(1, 1, 3, 64, 0, 0, 0, no_less(1, 0, true));
+                for (int stg : {2, 3, 1})
+                    for (int kbw : {64, 1})
+                        take(1, 1, stg, kbw, 0, 0, 0, any);
+            }
+            for (int stg : {2, 1})
+                for (int kbw : {64, 1})
+                    take(2, 1, stg, kbw, 0, 0, 0, any);
         }
         if (x3) {
             // the rest in shared memory, then (N of about 100 and more) A in tensor memory, one
@@ -2048,6 +2093,8 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
             for (int stg : {1, 2})
                 for (int kbw : {64, 1})
                     take(geo && !node ? 3 : 2, 1, stg, kbw, 0, 1, 0, any);
+            if (N <= 104)  // (one stage of wide K-blocks: N = 100, F = 3 370 us, two of narrow ones 472)
+                take(3, 1, 1, 64, 32, 0, 1, any);
             for (int stg : {2, 1})
                 for (int kbw : {64, 1})
                     take(2, 1, stg, kbw, 32, 0, 1, any);

@@ -25,9 +25,9 @@ def test_column_blocks_bit_exact(N, F, layout, tile_e):
     D = rng.integers(-8, 9, (F, N, N)).astype(np.float32)
     u = rng.integers(-8, 9, (E, N)).astype(np.float32)
     k = lc.Kernel()
-    v = lc.variant_default(k, E, N, F, layout, "fp32")
-    v.tile_e = tile_e
-    assert lc.variant_dict(v)["engine"] == "ksplit"
+    v = lc.Variant(engine="ksplit", layout=layout, precision="fp32", tile_e=tile_e, elems_per_thread=8, split_i=8,
+                   unroll=16, prefetch_smem=1, stages=1)
+    assert lc.variant_validate(k, E, N, F, v) == 0
     uu = u if layout == "elem" else u.T
     out = lc.contract(k, v, torch.from_numpy(D).cuda(), torch.from_numpy(np.ascontiguousarray(uu)).cuda())
     torch.cuda.synchronize()
