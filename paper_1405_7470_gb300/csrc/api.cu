@@ -2059,7 +2059,11 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
                     take(u, 1, 2, 1, 0, 0, 0, roomy);
             }
             if (N > 64 && N < 96 && F > 1)
-                take(u, 1, 3, 64, 0, 0, 0, no_less(u, 0, false));
+                // (equal blocks, or no more of them: N = 84, F = 4 305 us with two stages, 280 with three; for
+                // three operators from N = 80: N = 77 150 against 161, N = 84 153 against 132)
+                take(u, 1, 3, 64, 0, 0, 0, [F, N, keeps = no_less(u, 0, false)](const TcArgs &t) {
+                    return keeps(t) || (F % t.G == 0 && (F % 2 == 0 || N >= 80));
+                });
             for (int stg : {2, 3, 1})
                 for (int kbw : {64, 1})
                     take(u, 1, stg, kbw, 0, 0, 0, any);
