@@ -89,6 +89,14 @@ size_t smem_optin_limit()
     return (size_t)n;
 }
 
+cudaError_t allow_smem(const void *fn)
+{
+    const size_t limit = smem_optin_limit();
+    if (limit == 0)
+        return cudaErrorInvalidDevice;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit);
+}
+
 int current_cc(int *major, int *minor)
 {
     int dev = 0;
@@ -3117,7 +3125,7 @@ lc_status lc_grouped_plan_create(const lc_kernel *kh, const lc_variant *v, const
     if (e == cudaSuccess)
         e = cudaStreamSynchronize(s);
     if (e == cudaSuccess && fn)
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.smem);
+        e = allow_smem(fn);
     if (e != cudaSuccess)
         return cuda_fail(e);
     lc_grouped_plan *plan = new (std::nothrow) lc_grouped_plan;
@@ -3164,7 +3172,7 @@ lc_status lc_grouped_plan_create(const lc_kernel *kh, const lc_variant *v, const
     for (const TcLaunch &L : A.tcl)
         plan->nsegs += L.grid;
     plan->layout = v->layout;
-    // shared-memory sizes, before any capture
+    // shared-memory limits, before any capture
     for (const KsLaunch &L : A.ks) {
         st = ks_launch(L.a, v->layout, L.bm, L.bk, 0, s, true);
         if (st != LC_OK) {

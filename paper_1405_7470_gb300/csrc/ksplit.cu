@@ -393,7 +393,7 @@ lc_status ks_launch(const KsArgs &a, int layout, int bm, int bk, int grid, cudaS
     const size_t smem = ks_smem_bytes(a.Kp, bm, bk, a.bn, a.ubufs);
     cudaError_t e = cudaSuccess;
     if (set_attr) {
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_smem(fn);
         if (e != cudaSuccess)
             return cuda_fail(e);
     }

@@ -120,7 +120,7 @@ struct KsArgs {
     int vec_u;         // node-major: 16-byte copies of u rows (E % 4 == 0)
     int vec_out;       // 16-byte output stores (element-major: N % 4 == 0; node-major: E % 4 == 0)
 };
-// set_attr: set the instance's shared-memory size first; grid <= 0: only that.
+// set_attr: raise the instance's shared-memory limit first; grid <= 0: only that.
 lc_status ks_launch(const KsArgs &a, int layout, int bm, int bk, int grid, cudaStream_t s, bool set_attr = true);
 size_t ks_smem_bytes(int Kp, int bm, int bk, int bn, int ubufs);
 int ks_block_cols(int C, int bm);
@@ -243,6 +243,11 @@ lc_status cuda_fail(cudaError_t e);
 size_t smem_optin_limit();
 
 // SIMT launchers (one per element type / layout translation unit).
+// Let kernel `fn` be launched with any plan's dynamic shared memory.  Always the device's limit, not one
+// plan's size: the attribute belongs to the function, so a smaller plan on the same instance (another
+// thread's, or any call between a grouped plan's creation and its run) would make the larger plan's
+// launch fail.  (No kernel that uses it has static shared memory, which counts against the limit.)
+cudaError_t allow_smem(const void *fn);
 lc_status simt_launch_f32_elem(const SimtArgs &a, const SimtGeom &g, int unroll, int prefetch,
                                cudaStream_t s);
 lc_status simt_launch_f32_node(const SimtArgs &a, const SimtGeom &g, int unroll, int prefetch,

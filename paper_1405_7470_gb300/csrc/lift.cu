@@ -290,7 +290,7 @@ lc_status lift_launch(const LiftArgs &a, int grid, cudaStream_t s)
                                           : reinterpret_cast<void *>(&lift_kernel<false, 128>))
                            : (a.halo >= 0 ? reinterpret_cast<void *>(&lift_kernel<true, 64>)
                                           : reinterpret_cast<void *>(&lift_kernel<false, 64>));
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(fn);
     if (e != cudaSuccess)
         return cuda_fail(e);
     // a persistent grid no larger than the CTAs that are resident at once (shared memory may

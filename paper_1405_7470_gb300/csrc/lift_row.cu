@@ -439,7 +439,7 @@ lc_status lift_row_launch(const LiftArgs &a, int ept, int grid, size_t smem, cud
     void *fn = lift_row_fn(lift_row_half(a.M), ept);
     if (!fn)
         return LC_ERR_INVALID_VARIANT;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(fn);
     if (e != cudaSuccess)
         return cuda_fail(e);
     LiftArgs args = a;

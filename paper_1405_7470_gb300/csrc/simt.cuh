@@ -442,7 +442,7 @@ static lc_status simt_launch_impl(const SimtArgs &a, const SimtGeom &g, int unro
     else if (g.RE == 2 * V && g.RC == 2 * V) fn = simt_pick_unr<T, LAYOUT, 2 * V, 2 * V>(unroll, prefetch);
     if (!fn)
         return LC_ERR_INVALID_VARIANT;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+    cudaError_t e = allow_smem(fn);
     if (e != cudaSuccess)
         return cuda_fail(e);
     SimtArgs args = a;

@@ -277,7 +277,7 @@ lc_status row_launch(const SimtArgs &a, int layout, int ept, int grid, int threa
                    : (ept == 4 ? row_fn<LC_LAYOUT_ELEM_MAJOR, 4>(np) : row_fn<LC_LAYOUT_ELEM_MAJOR, 2>(np));
     if (!fn)
         return LC_ERR_INVALID_VARIANT;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(fn);
     if (e != cudaSuccess)
         return cuda_fail(e);
     SimtArgs args = a;

@@ -1155,10 +1155,10 @@ __global__ void __launch_bounds__(864, 1) tc_grouped_kernel(const __grid_constan
     tc_body<LAYOUT, NT, 8, 0, ATM>(P.g[m.x], m.y, m.z, m.w);
 }
 
-// Set the shared-memory size of one kernel instance and launch it.
+// Raise the shared-memory limit of one kernel instance and launch it.
 static inline lc_status tc_launch_fn(void *fn, const TcArgs &a, int grid, cudaStream_t s)
 {
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.smem_bytes);
+    cudaError_t e = allow_smem(fn);
     if (e != cudaSuccess)
         return cuda_fail(e);
     if (grid <= 0)

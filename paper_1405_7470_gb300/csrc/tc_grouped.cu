@@ -22,7 +22,7 @@ lc_status tc_grouped_launch(const TcGroupedParams &P, int layout, int nterms, in
     void *fn = fns[layout == LC_LAYOUT_NODE_MAJOR][nterms == 3 ? (atm ? 2 : 1) : 0];
     if (fn_out)
         *fn_out = fn;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(fn);
     if (e != cudaSuccess)
         return cuda_fail(e);
     if (grid <= 0)
