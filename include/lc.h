@@ -418,7 +418,11 @@ lc_status lc_grouped_workspace_size(const lc_kernel *k, const lc_variant *v, con
  * FP32 SIMT variant: every group gets a SIMT tile shape with the same CTA size; all
  * (group, tile) work is cut into one contiguous range per CTA, balanced by estimated
  * cost.  The variant gives the register block (elems_per_thread, split_i), unroll (1 or
- * 4), prefetch_smem, stages and ctas_per_sm.
+ * 4), prefetch_smem, stages and ctas_per_sm.  Groups of N >= 96 run after it as one K-split
+ * launch each (tiles of 128 elements, j chunks of 16, one u buffer).  The other two kinds of
+ * descriptor that lc_variant_default gives for N >= 13 are taken too: whole rows in registers
+ * (unroll 8 with prefetch_smem 1) runs as the tiles the launch has for the layout, and a K-split
+ * descriptor serves the groups of N >= 64, one launch each, beside those tiles for the others.
  * Tensor-core variant (TCGEN05, BF16 or BF16X3, at most 16 groups): each group that has
  * a tensor-core plan (lc_variant_validate's rules; the epilogue works in 8-column chunks)
  * for the variant, or else for the first of its changes "stages = 1", "the other K-block
@@ -457,9 +461,11 @@ lc_status lc_grouped_plan_info(const lc_grouped_plan *plan, int32_t *grid, int32
 
 /*
  * The descriptor that serves group `group` (0-based, < ngroups) of a plan: the variant as
- * given (SIMT plans; tensor-core groups that have a plan for it), the tensor-core variant
- * the planner fell back to for that group, or the FP32 SIMT descriptor of the groups
- * without a tensor-core plan.  Errors: LC_ERR_INVALID_ARGUMENT.
+ * given (SIMT plans; tensor-core groups that have a plan for it), the K-split descriptor of a
+ * group with a launch of its own, the tiles that stand in for the variant (unroll 8 or K-split,
+ * see lc_grouped_plan_create), the tensor-core variant the planner chose for that group, or the
+ * FP32 SIMT descriptor of the groups without a tensor-core plan.
+ * Errors: LC_ERR_INVALID_ARGUMENT.
  */
 lc_status lc_grouped_plan_group(const lc_grouped_plan *plan, int32_t group, lc_variant *v);
 

@@ -2432,6 +2432,7 @@ namespace lc {
 struct KsLaunch {
     KsArgs a;
     int grid, bm, bk, group;
+    lc_variant v;
 };
 
 // One plain tensor-core launch of a tensor-core grouped plan: a large group with its own default
@@ -2868,7 +2869,7 @@ struct GroupedPlanAll {
     GroupedPlanTc T;
     std::vector<lc_group> simt_groups;
     std::vector<int> simt_gi;  // their indices among the caller's groups
-    lc_variant simt_v, ks_v, tcl_v;
+    lc_variant simt_v, tcl_v;  // the descriptors of the SIMT launch and of the fallback tensor launches
     std::vector<KsLaunch> ks;
     std::vector<TcLaunch> tcl;
     bool has_simt = false;
@@ -2877,9 +2878,9 @@ struct GroupedPlanAll {
 
 // The K-split descriptor for the groups of a grouped plan that run as their own K-split
 // launch: tensor-core plans' groups without any tensor-core plan (N above 128 for three
-// terms), FP32 plans' groups of N >= 96 (tiles of 128 elements, j chunks of 16, one u buffer:
-// the fastest measured for N = 120 and 165).
-static lc_variant grouped_ks_fallback(const lc_variant *v)
+// terms), FP32 plans' groups of N >= 96 (tiles of 128 elements, j chunks of 16 or 8 as the default
+// has them, one u buffer: the fastest measured for N = 120 and 165).
+static lc_variant grouped_ks_fallback(const lc_variant *v, const lc_group &G)
 {
     lc_variant s;
     memset(&s, 0, sizeof s);
@@ -2938,9 +2939,34 @@ static lc_status grouped_add_ks(const Kernel &K, const lc_variant &kv, const lc_
     L.bm = r.ks_bm;
     L.bk = r.ks_bk;
     L.group = gi;
+    L.v = kv;
     ks.push_back(L);
     *added = true;
     return LC_OK;
+}
+
+// Descriptors the default gives that the persistent SIMT launch does not run itself: the row
+// kernel's (unroll 8) and the K-split engine's.  The groups then run in the register blocks that
+// are the fastest of that launch per layout: element-major 4 x 8 with j unrolled 4 times,
+// node-major 8 x 4 up to N = 24, 8 x 8 up to N = 40, 4 x 8 above.
+static lc_variant grouped_simt_tiles(const lc_variant *v, const lc_group *groups, int ng)
+{
+    lc_variant s = *v;
+    const bool ks = v->engine == LC_ENGINE_KSPLIT;
+    if (!ks && !(v->engine == LC_ENGINE_SIMT && v->precision == LC_PREC_FP32 && v->unroll == 8 && v->prefetch_smem == 1))
+        return s;
+    int most = 0;
+    for (int gi = 0; gi < ng; ++gi)
+        most = std::max(most, (int)groups[gi].N);
+    const bool node = v->layout == LC_LAYOUT_NODE_MAJOR;
+    s.engine = LC_ENGINE_SIMT;
+    s.elems_per_thread = node && most <= 40 ? 8 : 4;
+    s.split_i = node && most <= 24 ? 4 : 8;
+    s.unroll = node && most > 24 ? 1 : 4;
+    s.tile_e = 64;  // (each group gets its own)
+    s.prefetch_smem = 1;
+    s.stages = 2;
+    return s;
 }
 
 static lc_status grouped_plan_all(const Kernel &K, const lc_variant *v, const lc_group *groups, int ng,
@@ -2949,18 +2975,25 @@ static lc_status grouped_plan_all(const Kernel &K, const lc_variant *v, const lc
     if (!v || v->struct_size != sizeof(lc_variant) || !groups || ng <= 0)
         return LC_ERR_INVALID_ARGUMENT;
     if (v->engine != LC_ENGINE_TCGEN05) {
-        // FP32: the groups of N >= 96 (where the K-split kernel, which streams D^T in chunks,
-        // is the library's default) run as one K-split launch each after the persistent launch
-        lc_status st = grouped_plan_host(K, v, groups, ng, A.S);  // validates the descriptor
+        // FP32: large groups run as one K-split launch each (D^T streamed in chunks) after the
+        // persistent launch: those of N >= 96, or, with a K-split descriptor, of N >= 64 with that
+        // descriptor (below, its columns are mostly padding)
+        const bool ks = v->engine == LC_ENGINE_KSPLIT;
+        if (ks && (v->precision != LC_PREC_FP32 || v->tail_free))
+            return LC_ERR_INVALID_VARIANT;
+        A.simt_v = grouped_simt_tiles(v, groups, ng);
+        lc_status st = grouped_plan_host(K, &A.simt_v, groups, ng, A.S);  // validates the descriptor
         if (st != LC_OK)
             return st;
         if (v->precision == LC_PREC_FP32) {
-            A.ks_v = grouped_ks_fallback(v);
             for (int gi = 0; gi < ng; ++gi) {
                 const lc_group &G = groups[gi];
                 bool added = false;
-                if (G.E > 0 && G.N >= 96) {
-                    st = grouped_add_ks(K, A.ks_v, G, gi, A.ks, &added);
+                Resolved r;
+                if (ks && (st = resolve(K, G.E, G.N, G.F, v, r, true)) != LC_OK)
+                    return st;  // the descriptor has to be valid for every group
+                if (G.E > 0 && G.N >= (ks ? 64 : 96)) {
+                    st = grouped_add_ks(K, ks ? *v : grouped_ks_fallback(v, G), G, gi, A.ks, &added);
                     if (st != LC_OK)
                         return st;
                 }
@@ -2972,7 +3005,7 @@ static lc_status grouped_plan_all(const Kernel &K, const lc_variant *v, const lc
             if (!A.ks.empty()) {
                 A.S = GroupedPlanHost();
                 if (!A.simt_groups.empty()) {
-                    st = grouped_plan_host(K, v, A.simt_groups.data(), (int)A.simt_groups.size(), A.S);
+                    st = grouped_plan_host(K, &A.simt_v, A.simt_groups.data(), (int)A.simt_groups.size(), A.S);
                     if (st != LC_OK)
                         return st;
                 }
@@ -2990,7 +3023,6 @@ static lc_status grouped_plan_all(const Kernel &K, const lc_variant *v, const lc
     // the rest: three terms, one tensor-core launch each with the A terms in tensor memory
     // where that plan resolves; else one K-split launch each; else (no K-split plan) the SIMT
     // grouped launch
-    A.ks_v = grouped_ks_fallback(v);
     A.tcl_v = grouped_tc_fallback(v);
     auto add_tc = [&](int gi, const lc_variant &tv) -> lc_status {
         const lc_group &G = groups[gi];
@@ -3029,7 +3061,7 @@ static lc_status grouped_plan_all(const Kernel &K, const lc_variant *v, const lc
                 continue;
         }
         bool added = false;
-        const lc_status sk = grouped_add_ks(K, A.ks_v, G, gi, A.ks, &added);
+        const lc_status sk = grouped_add_ks(K, grouped_ks_fallback(v, G), G, gi, A.ks, &added);
         if (sk != LC_OK)
             return sk;
         if (!added) {
@@ -3104,7 +3136,7 @@ lc_status lc_grouped_plan_create(const lc_kernel *kh, const lc_variant *v, const
     if (workspace_bytes < A.bytes)
         return LC_ERR_BUFFER_TOO_SMALL;
     const GroupedPlanHost &P = A.S;
-    const lc_variant *sv = v->engine == LC_ENGINE_TCGEN05 ? &A.simt_v : v;
+    const lc_variant *sv = &A.simt_v;
     void *fn = nullptr;
     if (A.has_simt) {
         fn = grouped_kernel_ptr(sv->layout, sv->elems_per_thread, sv->split_i, sv->unroll, sv->prefetch_smem);
@@ -3156,7 +3188,7 @@ lc_status lc_grouped_plan_create(const lc_kernel *kh, const lc_variant *v, const
         }
     }
     plan->ngroups = ngroups;
-    plan->group_variant.assign(ngroups, *v);
+    plan->group_variant.assign(ngroups, v->engine == LC_ENGINE_TCGEN05 ? *v : A.simt_v);
     if (v->engine == LC_ENGINE_TCGEN05) {
         for (int gi = 0; gi < ngroups; ++gi)
             plan->group_variant[gi] = A.T.gv[gi];
@@ -3164,7 +3196,7 @@ lc_status lc_grouped_plan_create(const lc_kernel *kh, const lc_variant *v, const
             plan->group_variant[gi] = A.simt_v;
     }
     for (const KsLaunch &L : A.ks)
-        plan->group_variant[L.group] = A.ks_v;
+        plan->group_variant[L.group] = L.v;
     for (const TcLaunch &L : A.tcl)
         plan->group_variant[L.group] = L.v;
     plan->ks = A.ks;
