@@ -205,13 +205,14 @@ struct LiftArgs {
     unsigned int *err;     // device error word: bit 1 set on an index out of range
 };
 lc_status lift_launch(const LiftArgs &a, int grid, cudaStream_t s);
-// Row kernel (lift_row.cu): warps a CTA, halo rows, shared memory, CTA tiles (0 warps: not for this shape)
+// Row kernel (lift_row.cu): warps a CTA, halo rows, shared memory, CTA tiles (0 warps: not for this shape,
+// or the tiled kernel is the faster one)
 struct LiftRowPlan {
     int ept, warps, halo, stage_s;
     size_t smem;
     long long tiles;
 };
-LiftRowPlan lift_row_plan(long long E, int N, int M, int Nf, int sms, size_t smem_cap);
+LiftRowPlan lift_row_plan(long long E, int N, int M, int Nf, bool accumulate, int sms, size_t smem_cap);
 lc_status lift_row_launch(const LiftArgs &a, int ept, int grid, size_t smem, cudaStream_t s);
 size_t lift_smem_bytes(int N, int M, int Nf, int halo, int nbuf, int te);
 int lift_threads(int N, int te);

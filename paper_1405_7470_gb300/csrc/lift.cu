@@ -396,11 +396,11 @@ lc_status lc_lift(const lc_kernel *kh, const lc_variant *v, const float *L, cons
     a.te = te;
     a.bulk_store = ((uintptr_t)out & 15u) == 0;
     a.err = error_word();
-    // The row kernel where its operands can be staged and it holds a row's fluxes (up to four faces and
-    // 64 face nodes); E = 2^21, degree 4: 325 us against 605.  Beyond that (degree 5: M = 84), with two
-    // staging buffers or tiles of 128, the tiled kernel.
+    // The row kernel where its operands can be staged, it holds a row's fluxes (up to four faces and
+    // 64 face nodes) and it is the faster one (lift_row_plan); E = 2^21, degree 4: 325 us against 605.
+    // Beyond that (degree 5: M = 84), with two staging buffers or tiles of 128, the tiled kernel.
     if (halo >= 0 && nbuf == 1 && te == 64) {
-        const LiftRowPlan p = lift_row_plan(E, N, a.M, Nf, sms, smem_optin_limit());
+        const LiftRowPlan p = lift_row_plan(E, N, a.M, Nf, accumulate != 0, sms, smem_optin_limit());
         if (p.warps > 0) {
             a.halo = p.halo;
             a.stage_s = p.stage_s;

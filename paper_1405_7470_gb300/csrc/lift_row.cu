@@ -390,13 +390,34 @@ static void *lift_row_fn(int mh, int ept)
     }
 }
 
+// Which of the two kernels is the faster one, measured over N = 8 to 128 and M = 12 to 64 with
+// neighbours up to 64 elements away (us, tiled -> rows in registers).  Rows of 32 or 64 values meet
+// in one bank (N = 64, M = 64, E = 300007: 116 -> 173).  Long rows leave few warps beside the window
+// (N = 50, M = 30: 70 -> 89; N = 40, M = 60: 91 -> 75, but 104 -> 144 with neighbours 200 away); a batch
+// of one or a few warps an SM waits for those warps' products (E = 4099: N = 27, M = 27 11.5 -> 12.2,
+// N = 35, M = 60 12.8 -> 11.4; E = 12000: N = 60, M = 60 20 -> 17).  Accumulating, the tiled kernel's
+// reads of out weigh more than all that (N = 60, M = 60, E = 300007: 1.6 times as long).
+static bool lift_row_faster(long long E, int N, int M, bool accumulate, int sms)
+{
+    if (N % 32 == 0)
+        return false;
+    if (accumulate)
+        return true;
+    const long long per_sm = E / sms;
+    if (M >= 40)
+        return N <= (per_sm < 32 ? 40 : per_sm < 96 ? 63 : per_sm < 512 ? 45 : 36);
+    return N <= (per_sm < 32 ? 24 : 36);
+}
+
 // Warps with a chunk each (the others only help to lay out L): the number that ends soonest, a tile
 // costing about its chunks and two more for what does not depend on them.  Scales are staged unless
 // that costs a warp.
-LiftRowPlan lift_row_plan(long long E, int N, int M, int Nf, int sms, size_t cap)
+LiftRowPlan lift_row_plan(long long E, int N, int M, int Nf, bool accumulate, int sms, size_t cap)
 {
     LiftRowPlan p{};
     if (Nf > 4 || M > kLiftRowMaxM || E < 1 || E >= 1ll << 30)  // (tile bounds are ints)
+        return p;
+    if (!lift_row_faster(E, N, M, accumulate, sms))
         return p;
     p.ept = E <= 96ll * sms ? 2 : lift_row_ept(lift_row_half(M));
     const int ch = 16 * p.ept;
