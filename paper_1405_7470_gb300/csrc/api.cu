@@ -1889,10 +1889,33 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
         // F = 1 23.3, 2 x 2 27.1, 4 x 4 25.4).
         const bool wide = N <= 12 && E >= 64 * 152;
         d.engine = LC_ENGINE_SIMT;
-        d.elems_per_thread = wide ? 4 : 2;
-        d.split_i = 2;
-        d.tile_e = wide ? 64 : 32;
         d.stages = 2;
+        // Where the columns do not fit one CTA's 512 threads, the blocks of whole operators they are cut
+        // into may be uneven, and the smaller ones idle: the first shape whose padded columns are within a
+        // fifth of the least (N = 20, F = 4, E = 187501: 2 x 2 in tiles of 32 takes 3 + 1 operators, 750 us,
+        // in tiles of 64 one each, 502; N = 32, F = 3, E = 97657 671 against 511).
+        struct Shape {
+            int re, rc, te;
+        };
+        const Shape shapes[] = {{wide ? 4 : 2, 2, wide ? 64 : 32}, {2, 2, 64}, {2, 4, 32}, {4, 2, 32}, {4, 4, 64}};
+        constexpr int NS = sizeof shapes / sizeof shapes[0];
+        long long cols[NS], least = 0;
+        for (int q = 0; q < NS; ++q) {
+            lc_variant c = d;
+            c.elems_per_thread = shapes[q].re;
+            c.split_i = shapes[q].rc;
+            c.tile_e = shapes[q].te;
+            Resolved r;
+            cols[q] = resolve(kh->k, E, N, F, &c, r, false) == LC_OK ? (long long)r.g.nchunks * r.g.CW : 0;
+            if (cols[q] > 0 && (least == 0 || cols[q] < least))
+                least = cols[q];
+        }
+        int pick = 0;
+        while (pick < NS - 1 && (cols[pick] == 0 || 5 * cols[pick] > 6 * least))
+            ++pick;
+        d.elems_per_thread = shapes[pick].re;
+        d.split_i = shapes[pick].rc;
+        d.tile_e = shapes[pick].te;
     } else if (precision == LC_PREC_FP32) {
         // Just above 64 two operators' D^T still fit beside two CTAs of the SIMT kernel, and their columns
         // pad badly (N = 66, F = 2 403 against 534 us, N = 77, F = 2 429 against 477; N = 66, F = 3 407

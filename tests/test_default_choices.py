@@ -1,0 +1,33 @@
+"""Choices of lc_variant_default that measured slower when made otherwise (no GPU needed: the plans
+a default descriptor resolves to)."""
+
+import pytest
+
+from paper_1405_7470_gb300 import lc
+
+
+@pytest.fixture(scope="module")
+def kernel():
+    from paper_1405_7470_gb300 import build
+    build()
+    return lc.Kernel()
+
+
+def default(kernel, E, N, F, layout, precision):
+    v = lc.variant_default(kernel, E, N, F, layout, precision)
+    return v, lc.variant_plan(kernel, E, N, F, v)
+
+
+@pytest.mark.parametrize("layout", ["elem", "node"])
+@pytest.mark.parametrize("N,F,E", [(20, 4, 187501), (20, 4, 40000), (32, 3, 97657), (24, 3, 173611), (28, 3, 35714),
+                                   (20, 1, 4096), (48, 1, 200000), (84, 2, 20000)])
+def test_fp64_blocks_of_even_width(kernel, layout, N, F, E):
+    """The columns of all blocks together, padding included, stay within a quarter of F N."""
+    v, p = default(kernel, E, N, F, layout, "fp64")
+    width = p["threads"] // (v.tile_e // v.elems_per_thread) * v.split_i
+    assert p["column_blocks"] * width <= 1.25 * F * N
+
+
+def test_fp64_small_batch_keeps_small_tiles(kernel):
+    v, _ = default(kernel, 4096, 20, 1, "elem", "fp64")
+    assert (v.elems_per_thread, v.split_i, v.tile_e) == (2, 2, 32)
