@@ -1959,7 +1959,7 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
                 return LC_OK;
             }
         }
-        // SIMT.  N <= 40: the row kernel (unroll 8: the whole rows of u in registers); E = 2^21,
+        // SIMT.  13 <= N <= 40: the row kernel (unroll 8: the whole rows of u in registers); E = 2^21,
         // F = 3: N = 35 494 -> 351 us element-major, 486 -> 356 node-major; N = 20 280 -> 121 and
         // 228 -> 142; E = 4099, N = 35: 14.7 -> 10.6 and 21 -> 11.  Above: tiles, two CTAs per SM, the
         // u tile staged by bulk copies two tiles ahead; element-major 4 x 8 register blocks with
@@ -1971,7 +1971,16 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
         d.stages = 2;
         d.elems_per_thread = 4;
         d.split_i = 8;
-        if (N <= 40) {
+        if (N < 13) {
+            // (more columns than a warp of the warp engine takes) node-major rows that the bulk copies can
+            // fetch: 8 x 4 blocks in tiles of 128 while there are few columns (N = 4, F = 6, E = 357140:
+            // 19.4 against 27.6 us; N = 10, F = 8: 26 against 20)
+            const bool tall = layout == LC_LAYOUT_NODE_MAJOR && E % 4 == 0 && F * N <= 60;
+            d.elems_per_thread = tall ? 8 : 4;
+            d.split_i = tall ? 4 : 8;
+            d.tile_e = tall ? 128 : 64;
+            d.unroll = tall || N < 8 ? 4 : 8;
+        } else if (N <= 40) {
             d.tile_e = 64;
             d.unroll = 8;
         } else if (layout == LC_LAYOUT_ELEM_MAJOR) {

@@ -31,3 +31,13 @@ def test_fp64_blocks_of_even_width(kernel, layout, N, F, E):
 def test_fp64_small_batch_keeps_small_tiles(kernel):
     v, _ = default(kernel, 4096, 20, 1, "elem", "fp64")
     assert (v.elems_per_thread, v.split_i, v.tile_e) == (2, 2, 32)
+
+
+@pytest.mark.parametrize("layout,N,F,E,want", [
+    ("node", 4, 6, 357140, (8, 4, 128, 4)), ("node", 6, 8, 46296, (8, 4, 128, 4)), ("node", 4, 6, 357141, (4, 8, 64, 4)),
+    ("node", 10, 8, 111108, (4, 8, 64, 8)), ("elem", 4, 6, 357140, (4, 8, 64, 4)), ("elem", 8, 8, 138888, (4, 8, 64, 8))])
+def test_fp32_few_nodes_many_operators(kernel, layout, N, F, E, want):
+    """Up to N = 12 with more columns than the warp engine takes: register blocks, tile and unrolling."""
+    v, _ = default(kernel, E, N, F, layout, "fp32")
+    assert lc.variant_dict(v)["engine"] == "simt"
+    assert (v.elems_per_thread, v.split_i, v.tile_e, v.unroll) == want
