@@ -1921,7 +1921,11 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
         // pad badly (N = 66, F = 2 403 against 534 us, N = 77, F = 2 429 against 477; N = 66, F = 3 407
         // against 447; at N = 70, F = 3 and N = 66, F = 4 the K-split kernel is ahead).
         const bool tiles = N > 64 && N < 80 && (F == 2 || (N < 70 && F < 4));
-        if (N >= 64 && !tiles) {
+        // Few elements and many columns: a K-split CTA walks all the column blocks of its tile, so most
+        // SMs would idle; the SIMT kernel's column blocks are CTAs of their own (8 x 4 blocks in tiles of
+        // 128; N = 95, F = 8, E = 818: 20 against 53 us element-major, 34 against 47 node-major).
+        const bool few = N > 64 && N < 96 && F >= 6 && E <= 1536;
+        if (N >= 64 && !tiles && !few) {
             // large N: the K-split kernel (D^T streamed in chunks of 16 j) against the SIMT
             // kernel holding all of D^T: N = 64, F = 3, E = 2^19 392 against 476 us element-major,
             // 318 against 345 node-major; N = 84, F = 4, E = 2^20 1565 against 1746 and 1342
@@ -1980,6 +1984,11 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
             d.split_i = tall ? 4 : 8;
             d.tile_e = tall ? 128 : 64;
             d.unroll = tall || N < 8 ? 4 : 8;
+        } else if (few) {
+            d.elems_per_thread = 8;
+            d.split_i = 4;
+            d.tile_e = 128;
+            d.unroll = 4;
         } else if (N <= 40) {
             d.tile_e = 64;
             d.unroll = 8;

@@ -41,3 +41,16 @@ def test_fp32_few_nodes_many_operators(kernel, layout, N, F, E, want):
     v, _ = default(kernel, E, N, F, layout, "fp32")
     assert lc.variant_dict(v)["engine"] == "simt"
     assert (v.elems_per_thread, v.split_i, v.tile_e, v.unroll) == want
+
+
+@pytest.mark.parametrize("layout", ["elem", "node"])
+@pytest.mark.parametrize("N,F,E,engine", [(95, 8, 818, "simt"), (66, 8, 1178, "simt"), (84, 6, 1536, "simt"),
+                                          (84, 6, 1537, "ksplit"), (84, 5, 900, "ksplit"), (64, 8, 1214, "ksplit"),
+                                          (96, 8, 800, "ksplit")])
+def test_fp32_few_elements_many_columns(kernel, layout, N, F, E, engine):
+    """K-split CTAs walk their tile's column blocks: with few tiles of many columns the SIMT kernel, whose
+    column blocks are CTAs, uses more of the GPU."""
+    v, p = default(kernel, E, N, F, layout, "fp32")
+    assert lc.variant_dict(v)["engine"] == engine
+    if engine == "simt":
+        assert p["column_blocks"] >= F
