@@ -1937,7 +1937,7 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
             k.tile_e = (E + 127) / 128 < 152 ? 64 : 128;
             k.elems_per_thread = 8;
             k.split_i = 8;
-            k.unroll = 16;
+            k.unroll = ks_chunk(N, F, k.tile_e);
             k.prefetch_smem = 1;
             k.stages = 1;
             if (lc_variant_validate(kh, E, N, F, &k) == LC_OK) {
@@ -2932,7 +2932,7 @@ static lc_variant grouped_ks_fallback(const lc_variant *v, const lc_group &G)
     s.tile_e = 128;
     s.elems_per_thread = 8;
     s.split_i = 8;
-    s.unroll = 16;
+    s.unroll = ks_chunk(G.N, G.F, 128);
     s.prefetch_smem = 1;
     s.stages = 1;
     return s;

@@ -356,6 +356,17 @@ int ks_block_cols(int C, int bm)
     return width[best];
 }
 
+// Length of the j chunks: 16, but 8 where two CTAs of 128 elements then fit an SM and with 16 only one
+// (N = 177 to 200; N = 200, F = 1, E = 100001: 309 -> 282 us).
+int ks_chunk(int N, int F, int bm)
+{
+    if (bm != 128)
+        return 16;
+    const size_t two = 232448 / 2 - 1024;  // (1 KB reserved per CTA)
+    auto bytes = [&](int bk) { return ks_smem_bytes((N + bk - 1) / bk * bk, bm, bk, ks_block_cols(F * N, bm), 1); };
+    return bytes(16) > two && bytes(8) <= two ? 8 : 16;
+}
+
 int ks_threads(int bm, int bn) { return (bm / 8) * (bn / 8); }
 
 size_t ks_smem_bytes(int Kp, int bm, int bk, int bn, int ubufs)

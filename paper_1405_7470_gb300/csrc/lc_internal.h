@@ -124,6 +124,7 @@ struct KsArgs {
 lc_status ks_launch(const KsArgs &a, int layout, int bm, int bk, int grid, cudaStream_t s, bool set_attr = true);
 size_t ks_smem_bytes(int Kp, int bm, int bk, int bn, int ubufs);
 int ks_block_cols(int C, int bm);
+int ks_chunk(int N, int F, int bm);
 int ks_threads(int bm, int bn);
 
 // Tensor-core kernel (tcgen05): one column block of G operators per CTA.

@@ -54,3 +54,13 @@ def test_fp32_few_elements_many_columns(kernel, layout, N, F, E, engine):
     assert lc.variant_dict(v)["engine"] == engine
     if engine == "simt":
         assert p["column_blocks"] >= F
+
+
+@pytest.mark.parametrize("layout", ["elem", "node"])
+@pytest.mark.parametrize("N,F,chunk", [(176, 1, 16), (177, 3, 8), (185, 2, 8), (200, 3, 8), (201, 3, 16), (120, 3, 16)])
+def test_ksplit_chunks_leave_room_for_two_ctas(kernel, layout, N, F, chunk):
+    """Chunks of 8 where two CTAs of 128 elements then share an SM's 228 KB and with 16 they would not."""
+    v, p = default(kernel, 400000, N, F, layout, "fp32")
+    assert (v.tile_e, v.unroll) == (128, chunk)
+    if N <= 200:
+        assert 2 * (p["smem_bytes"] + 1024) <= 228 * 1024
