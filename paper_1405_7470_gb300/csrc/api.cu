@@ -2096,13 +2096,16 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
                     take(4, 1, stg, kbw, 0, 0, 0, any);
         } else if (!x3 && !node) {
             // BF16: many warps up to N = 48, fewer above.  Three stages where two A buffers and two
-            // slots fit beside them (N = 20, F = 1 229 -> 207 us, N = 50, F = 1 143 -> 128), and between
-            // N = 64 and 96 for several operators (N = 84, F = 3 153 -> 132, N = 70, F = 4 201 -> 144;
-            // for one 128 against 142); narrow K-blocks where only they leave room for both (N = 35,
+            // slots fit beside them (N = 20, F = 1 229 -> 207 us, N = 50, F = 1 143 -> 128) and the output
+            // is narrow (from 88 columns on two stages are as fast or faster: N = 47, F = 2 70.5 against
+            // 75.6, N = 35, F = 3 70.5 against 77.6, N = 29, F = 3 72.9 both), and between N = 64 and 96
+            // for several operators (N = 84, F = 3 153 -> 132, N = 70, F = 4 201 -> 144; for one 128
+            // against 142); narrow K-blocks where only they leave room for both (N = 35,
             // F = 4 140 -> 132)
             const int u = N <= 48 ? 3 : 2;
             if (N <= 64) {
-                take(u, 1, 3, 64, 0, 0, 0, roomy);
+                if (F * N < 88)
+                    take(u, 1, 3, 64, 0, 0, 0, roomy);
                 take(u, 1, 2, 64, 0, 0, 0, roomy);
                 if (N <= 48)
                     take(u, 1, 2, 1, 0, 0, 0, roomy);

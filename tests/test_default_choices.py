@@ -64,3 +64,11 @@ def test_ksplit_chunks_leave_room_for_two_ctas(kernel, layout, N, F, chunk):
     assert (v.tile_e, v.unroll) == (128, chunk)
     if N <= 200:
         assert 2 * (p["smem_bytes"] + 1024) <= 228 * 1024
+
+
+@pytest.mark.parametrize("N,F,stages", [(27, 4, 2), (33, 3, 2), (35, 3, 2), (44, 2, 2), (47, 2, 2), (29, 3, 3), (20, 4, 3),
+                                        (50, 1, 3)])
+def test_bf16_element_major_stages(kernel, N, F, stages):
+    """A third stage for narrow outputs only."""
+    v, _ = default(kernel, 700000, N, F, "elem", "bf16")
+    assert v.stages == stages
