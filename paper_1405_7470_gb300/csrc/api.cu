@@ -2123,8 +2123,9 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
             // BF16, node-major.  Up to N = 64: three stages, but with many columns two stages and
             // more threads a row (N = 64, F = 3 147 -> 136 us, N = 56, F = 4 174 -> 159; N = 44, F = 3
             // 139 against 143).  Up to N = 96: few warps, three stages unless they cost an A
-            // buffer or an operator of the block (N = 77, F = 3 181 against 143 with two).  Above: two stages, two threads
-            // (N = 112, F = 4 165 against 280 with one and three stages).
+            // buffer or an operator of the block (N = 77, F = 3 181 against 143 with two); for three
+            // operators below N = 80, two threads and two stages (N = 65 92.7 -> 77.0, N = 73 78 -> 75).
+            // Above: two stages, two threads (N = 112, F = 4 165 against 280 with one and three stages).
             if (N <= 64 && F * N >= 140)
                 for (int kbw : {64, 1})
                     take(4, 1, 2, kbw, 0, 0, 0, any);
@@ -2133,6 +2134,8 @@ lc_status lc_variant_default(const lc_kernel *kh, int64_t E, int32_t N, int32_t 
                     for (int kbw : {64, 1})
                         take(3, 1, stg, kbw, 0, 0, 0, any);
             if (N <= 96) {
+                if (F == 3 && N < 80)
+                    take(2, 1, 2, 64, 0, 0, 0, any);
                 take(1, 1, 3, 64, 0, 0, 0, no_less(1, 0, true));
                 for (int stg : {2, 3, 1})
                     for (int kbw : {64, 1})

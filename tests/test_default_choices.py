@@ -72,3 +72,10 @@ def test_bf16_element_major_stages(kernel, N, F, stages):
     """A third stage for narrow outputs only."""
     v, _ = default(kernel, 700000, N, F, "elem", "bf16")
     assert v.stages == stages
+
+
+@pytest.mark.parametrize("N,F,want", [(65, 3, (2, 2)), (66, 3, (2, 2)), (79, 3, (2, 2)), (66, 2, (1, 3)), (84, 3, (1, 2))])
+def test_bf16_node_major_three_operators(kernel, N, F, want):
+    """Two threads a row and two stages for three operators between N = 65 and 79."""
+    v, _ = default(kernel, 378784, N, F, "node", "bf16")
+    assert (v.unroll, v.stages) == want
