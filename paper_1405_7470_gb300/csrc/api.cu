@@ -1311,8 +1311,8 @@ static lc_status resolve(const Kernel &K, long long E, int N, int F, const lc_va
         // takes tensor-memory A where no shared-memory plan fits (N above about 100)
         const bool tm_first = v->a_operand == 2 || (v->a_operand == 0 && NT == 1);
         // (node-major rows that are not 16-byte aligned need stage rows of 132 values; where that
-        // does not fit, the tiles are read from global memory)
-        for (int shifted = node && E % 4 != 0 ? 1 : 0; shifted >= 0 && !found; --shifted)
+        // does not fit, or no tile has a 132nd value, the tiles are read from global memory)
+        for (int shifted = node && E % 4 != 0 && E >= 132 ? 1 : 0; shifted >= 0 && !found; --shifted)
         for (int g = g_hi; g >= g_lo && !found; --g)
             for (int pass = 0; pass < 2 && !found; ++pass) {
                 const bool a_tm = tm_first ? pass == 0 : pass == 1;

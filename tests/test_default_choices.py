@@ -79,3 +79,15 @@ def test_bf16_node_major_three_operators(kernel, N, F, want):
     """Two threads a row and two stages for three operators between N = 65 and 79."""
     v, _ = default(kernel, 378784, N, F, "node", "bf16")
     assert (v.unroll, v.stages) == want
+
+
+@pytest.mark.parametrize("E", [1, 5, 127, 130, 131])
+def test_short_node_major_rows_keep_the_aligned_plan(kernel, E):
+    """Rows off the 16-byte boundary with no 132nd value are never fetched in bulk: the wider stage rows
+    for that must not cost an operator of the block or an A buffer."""
+    for N, F in ((126, 3), (128, 4), (112, 4), (35, 3)):
+        for precision in ("bf16", "bf16x3"):
+            v, p = default(kernel, 128, N, F, "node", precision)
+            q = lc.variant_plan(kernel, E, N, F, v)
+            for key in ("ops_per_block", "a_buffers", "a_in_tmem", "smem_bytes"):
+                assert q[key] == p[key], (N, F, precision, key)
