@@ -73,7 +73,7 @@ __device__ __forceinline__ float lds_f32(uint32_t addr)
     return v;
 }
 
-template <int MH, int EPT>
+template <int MH, int EPT, bool LINES>  // LINES: M = 2 MH is a multiple of 32
 __global__ void __launch_bounds__(32 * kLiftRowWarps, 1) lift_row_kernel(LiftArgs a)
 {
     constexpr int CH = 16 * EPT;  // elements of a warp's chunk
@@ -238,45 +238,47 @@ __global__ void __launch_bounds__(32 * kLiftRowWarps, 1) lift_row_kernel(LiftArg
                     q[m] = 0;  // (padding: 2 MH - 8 < M)
                 far = max(far, (unsigned int)q[m]);
             }
-            unsigned int left = __ballot_sync(0xffffffffu, far >= (unsigned int)wn);
-            if (left != 0) {
-                parked = true;
-                if (MH % 16 == 0 && (M & 31) == 0) {
-                    // Index rows of whole 128-byte lines: lanes that each walk their own row meet in one bank,
-                    // and so they take the halves together, a row's half over neighbouring lanes (two where
-                    // 16 lanes cover it).  (N = 24, M = 64, E = 1000003, 1000 away: 619 -> 352 us; for other
-                    // M the rows in turn below are as fast or faster, degree 4 353 against 273.)
-                    left &= __ballot_sync(0xffffffffu, live);
-                    constexpr int P = MH <= 16 ? 2 : 1;
-                    const int sub = lane / (32 / P), m = lane % (32 / P);
-                    int *base = x < 2 ? vA : vB + (x / 2 - 1) * 32 * M;
-                    for (int o0 = 0; o0 < 32; o0 += 8 * P) {
-                        if ((left >> o0 & (0xffffffffu >> (32 - 8 * P))) == 0)
-                            continue;
-                        float v[8];
-                        int at[8];
-                        unsigned int outside = 0;
+            if constexpr (LINES) {
+                // Index rows of whole 128-byte lines: lanes that each walk their own row would meet in one
+                // bank, and so they take the far halves together, a row's half over neighbouring lanes (two
+                // where 16 lanes cover it).  (N = 24, M = 64, E = 1000003, 1000 away: 619 -> 352 us; for
+                // other M a row a lane is as fast or faster, degree 4 273 against 353.)
+                unsigned int left = __ballot_sync(0xffffffffu, far >= (unsigned int)wn);
+                parked = parked || left != 0;
+                left &= __ballot_sync(0xffffffffu, live);
+                constexpr int P = MH <= 16 ? 2 : 1;
+                const int sub = lane / (32 / P), m = lane % (32 / P);
+                int *base = x < 2 ? vA : vB + (x / 2 - 1) * 32 * M;
+                for (int o0 = 0; o0 < 32; o0 += 8 * P) {
+                    if ((left >> o0 & (0xffffffffu >> (32 - 8 * P))) == 0)
+                        continue;
+                    float v[8];
+                    int at[8];
+                    unsigned int outside = 0;
 #pragma unroll
-                        for (int k = 0; k < 8; ++k)
-                            if ((left >> (o0 + k * P) & ((1u << P) - 1u)) != 0) {
-                                const int o = o0 + k * P + sub;  // the lane whose half it is
-                                at[k] = ((x & 1) ? o ^ 16 : o) * M + (o >> 4) * MH + m;
-                                const int g = left >> o & 1u ? base[at[k]] : wb;
-                                v[k] = __int_as_float(0x7fc00000);
-                                if ((unsigned int)(g - wb) >= (unsigned int)wn) {
-                                    outside |= 1u << k;
-                                    if ((unsigned int)g < (unsigned int)(E * N))
-                                        v[k] = __ldg(a.u + g);
-                                    else
-                                        atomicOr(a.err, 2u);
-                                }
+                    for (int k = 0; k < 8; ++k)
+                        if ((left >> (o0 + k * P) & ((1u << P) - 1u)) != 0) {
+                            const int o = o0 + k * P + sub;  // the lane whose half it is
+                            at[k] = ((x & 1) ? o ^ 16 : o) * M + (o >> 4) * MH + m;
+                            const int g = left >> o & 1u ? base[at[k]] : wb;
+                            v[k] = __int_as_float(0x7fc00000);
+                            if ((unsigned int)(g - wb) >= (unsigned int)wn) {
+                                outside |= 1u << k;
+                                if ((unsigned int)g < (unsigned int)(E * N))
+                                    v[k] = __ldg(a.u + g);
+                                else
+                                    atomicOr(a.err, 2u);
                             }
+                        }
 #pragma unroll
-                        for (int k = 0; k < 8; ++k)
-                            if (outside >> k & 1u)
-                                base[at[k]] = __float_as_int(v[k]);
-                    }
-                } else if (live) {
+                    for (int k = 0; k < 8; ++k)
+                        if (outside >> k & 1u)
+                            base[at[k]] = __float_as_int(v[k]);
+                }
+                __syncwarp();
+            } else if (__any_sync(0xffffffffu, far >= (unsigned int)wn)) {
+                parked = true;
+                if (live) {
                     // eight at a time: their loads are in flight together
                     for (int mb = 0; mb < MH; mb += 8) {
                         float v[8];
@@ -404,35 +406,35 @@ __global__ void __launch_bounds__(32 * kLiftRowWarps, 1) lift_row_kernel(LiftArg
         bulk_wait0();
 }
 
-template <int MH>
+template <int MH, bool LINES = false>
 static void *lift_row_of(int ept)
 {
-    return ept == 2 ? reinterpret_cast<void *>(&lift_row_kernel<MH, 2>)
-                    : reinterpret_cast<void *>(&lift_row_kernel<MH, lift_row_ept(MH)>);
+    return ept == 2 ? reinterpret_cast<void *>(&lift_row_kernel<MH, 2, LINES>)
+                    : reinterpret_cast<void *>(&lift_row_kernel<MH, lift_row_ept(MH), LINES>);
 }
 
-static void *lift_row_fn(int mh, int ept)
+static void *lift_row_fn(int mh, int ept, bool lines)
 {
     switch (mh) {
     case 4: return lift_row_of<4>(ept);
     case 8: return lift_row_of<8>(ept);
     case 12: return lift_row_of<12>(ept);
-    case 16: return lift_row_of<16>(ept);
+    case 16: return lines ? lift_row_of<16, true>(ept) : lift_row_of<16>(ept);
     case 20: return lift_row_of<20>(ept);
     case 24: return lift_row_of<24>(ept);
     case 28: return lift_row_of<28>(ept);
-    case 32: return lift_row_of<32>(ept);
+    case 32: return lines ? lift_row_of<32, true>(ept) : lift_row_of<32>(ept);
     default: return nullptr;
     }
 }
 
 // Which of the two kernels is the faster one, measured over N = 8 to 128 and M = 12 to 64 with
 // neighbours up to 64 elements away (us, tiled -> rows in registers).  Rows of 32 or 64 values meet
-// in one bank (N = 64, M = 64, E = 300007: 116 -> 173).  Long rows leave few warps beside the window
-// (N = 50, M = 30: 70 -> 89; N = 40, M = 60: 91 -> 75, but 104 -> 144 with neighbours 200 away); a batch
-// of one or a few warps an SM waits for those warps' products (E = 4099: N = 27, M = 27 11.5 -> 12.2,
-// N = 35, M = 60 12.8 -> 11.4; E = 12000: N = 60, M = 60 20 -> 17).  Accumulating, the tiled kernel's
-// reads of out weigh more than all that (N = 60, M = 60, E = 300007: 1.6 times as long).
+// in one bank (N = 64, M = 64, E = 300007: 110 -> 167).  Long rows leave few warps beside the window
+// (N = 50, M = 30: 66 -> 84; N = 40, M = 60: 92 -> 74, but N = 37 104 -> 121 with neighbours 200 away); a
+// batch of one or a few warps an SM waits for those warps' products (E = 4099: N = 27, M = 27 5.9 ->
+// 6.3, N = 35, M = 60 8.8 -> 7.9; E = 12000: N = 60, M = 60 12.6 -> 11.0).  Accumulating, the tiled
+// kernel's reads of out weigh more than all that (N = 60, M = 60, E = 300007: 231 -> 142).
 static bool lift_row_faster(long long E, int N, int M, bool accumulate, int sms)
 {
     if (N % 32 == 0)
@@ -493,7 +495,7 @@ LiftRowPlan lift_row_plan(long long E, int N, int M, int Nf, bool accumulate, in
 
 lc_status lift_row_launch(const LiftArgs &a, int ept, int grid, size_t smem, cudaStream_t s)
 {
-    void *fn = lift_row_fn(lift_row_half(a.M), ept);
+    void *fn = lift_row_fn(lift_row_half(a.M), ept, a.M % 32 == 0);
     if (!fn)
         return LC_ERR_INVALID_VARIANT;
     cudaError_t e = allow_smem(fn);
