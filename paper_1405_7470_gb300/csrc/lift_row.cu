@@ -244,38 +244,40 @@ __global__ void __launch_bounds__(32 * kLiftRowWarps, 1) lift_row_kernel(LiftArg
                 // where 16 lanes cover it).  (N = 24, M = 64, E = 1000003, 1000 away: 619 -> 352 us; for
                 // other M a row a lane is as fast or faster, degree 4 273 against 353.)
                 unsigned int left = __ballot_sync(0xffffffffu, far >= (unsigned int)wn);
-                parked = parked || left != 0;
-                left &= __ballot_sync(0xffffffffu, live);
-                constexpr int P = MH <= 16 ? 2 : 1;
-                const int sub = lane / (32 / P), m = lane % (32 / P);
-                int *base = x < 2 ? vA : vB + (x / 2 - 1) * 32 * M;
-                for (int o0 = 0; o0 < 32; o0 += 8 * P) {
-                    if ((left >> o0 & (0xffffffffu >> (32 - 8 * P))) == 0)
-                        continue;
-                    float v[8];
-                    int at[8];
-                    unsigned int outside = 0;
+                if (left != 0) {
+                    parked = true;
+                    left &= __ballot_sync(0xffffffffu, live);
+                    constexpr int P = MH <= 16 ? 2 : 1;
+                    const int sub = lane / (32 / P), m = lane % (32 / P);
+                    int *base = x < 2 ? vA : vB + (x / 2 - 1) * 32 * M;
+                    for (int o0 = 0; o0 < 32; o0 += 8 * P) {
+                        if ((left >> o0 & (0xffffffffu >> (32 - 8 * P))) == 0)
+                            continue;
+                        float v[8];
+                        int at[8];
+                        unsigned int outside = 0;
 #pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        if ((left >> (o0 + k * P) & ((1u << P) - 1u)) != 0) {
-                            const int o = o0 + k * P + sub;  // the lane whose half it is
-                            at[k] = ((x & 1) ? o ^ 16 : o) * M + (o >> 4) * MH + m;
-                            const int g = left >> o & 1u ? base[at[k]] : wb;
-                            v[k] = __int_as_float(0x7fc00000);
-                            if ((unsigned int)(g - wb) >= (unsigned int)wn) {
-                                outside |= 1u << k;
-                                if ((unsigned int)g < (unsigned int)(E * N))
-                                    v[k] = __ldg(a.u + g);
-                                else
-                                    atomicOr(a.err, 2u);
+                        for (int k = 0; k < 8; ++k)
+                            if ((left >> (o0 + k * P) & ((1u << P) - 1u)) != 0) {
+                                const int o = o0 + k * P + sub;  // the lane whose half it is
+                                at[k] = ((x & 1) ? o ^ 16 : o) * M + (o >> 4) * MH + m;
+                                const int g = left >> o & 1u ? base[at[k]] : wb;
+                                v[k] = __int_as_float(0x7fc00000);
+                                if ((unsigned int)(g - wb) >= (unsigned int)wn) {
+                                    outside |= 1u << k;
+                                    if ((unsigned int)g < (unsigned int)(E * N))
+                                        v[k] = __ldg(a.u + g);
+                                    else
+                                        atomicOr(a.err, 2u);
+                                }
                             }
-                        }
 #pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        if (outside >> k & 1u)
-                            base[at[k]] = __float_as_int(v[k]);
+                        for (int k = 0; k < 8; ++k)
+                            if (outside >> k & 1u)
+                                base[at[k]] = __float_as_int(v[k]);
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
             } else if (__any_sync(0xffffffffu, far >= (unsigned int)wn)) {
                 parked = true;
                 if (live) {
