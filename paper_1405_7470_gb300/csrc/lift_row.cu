@@ -436,14 +436,16 @@ static void *lift_row_fn(int mh, int ept, bool lines)
 // (N = 50, M = 30: 66 -> 84; N = 40, M = 60: 92 -> 74, but N = 37 104 -> 121 with neighbours 200 away); a
 // batch of one or a few warps an SM waits for those warps' products (E = 4099: N = 27, M = 27 5.9 ->
 // 6.3, N = 35, M = 60 8.8 -> 7.9; E = 12000: N = 60, M = 60 12.6 -> 11.0).  Accumulating, the tiled
-// kernel's reads of out weigh more than all that (N = 60, M = 60, E = 300007: 231 -> 142).
+// kernel's reads of out weigh more than all that (N = 60, M = 60, E = 300007: 231 -> 142), and in small
+// batches more than the bank conflicts of N = 32 (M = 60, E = 14000: 13.0 -> 10.2; N = 64 14.3 -> 13.4,
+// but E = 9000 11.5 -> 12.2).
 static bool lift_row_faster(long long E, int N, int M, bool accumulate, int sms)
 {
+    const long long per_sm = E / sms;
     if (N % 32 == 0)
-        return false;
+        return N == 32 && accumulate && per_sm < 96;
     if (accumulate)
         return true;
-    const long long per_sm = E / sms;
     if (M >= 40)
         return N <= (per_sm < 32 ? 40 : per_sm < 96 ? 63 : per_sm < 512 ? 45 : 36);
     return N <= (per_sm < 32 ? 24 : 36);

@@ -24,7 +24,8 @@ def dev(*arrays):
     (30000, 50, 1, 30, False, True), (30000, 48, 3, 9, False, True), (4099, 27, 3, 9, False, True),
     (20000, 35, 4, 15, False, False), (4099, 35, 4, 15, False, False), (20000, 20, 4, 10, False, False),
     (4099, 20, 4, 10, False, False), (12000, 60, 4, 15, False, False), (20000, 64, 4, 16, True, True),
-    (4099, 27, 3, 9, True, False), (12000, 50, 1, 30, True, False)])
+    (4099, 27, 3, 9, True, False), (12000, 50, 1, 30, True, False), (12000, 32, 4, 15, True, False),
+    (12000, 64, 4, 15, True, True), (20000, 32, 4, 15, True, True)])
 def test_kernel_by_shape(E, N, Nf, Nfp, accumulate, tiled):
     """Both kernels' sums differ in their last bits (the tiled kernel adds m in order, the other one the
     halves of m apart), so the bits tell which one ran."""
