@@ -93,7 +93,7 @@ GROUPED_TC_CANDIDATES = [(64, 4, 1, 128, 1), (1, 4, 1, 128, 1), (64, 3, 1, 128, 
 # sources that decide each measured kernel's launch: the kernel, its helpers, the planner
 TC_SOURCES = ('tc.cu', 'tc.cuh', 'tma.cuh', 'lc_internal.h', 'api.cu')
 GEO_SOURCES = ('tc_geo.cu', 'tc.cuh', 'tma.cuh', 'lc_internal.h', 'api.cu')
-LIFT_SOURCES = ('lift.cu', 'tma.cuh', 'lc_internal.h', 'api.cu')
+LIFT_SOURCES = ('lift.cu', 'lift_row.cu', 'row.cuh', 'tma.cuh', 'lc_internal.h', 'api.cu')
 SAXPY_SOURCES = ('frontend.cu', 'lc_internal.h', 'api.cu')
 
 # DRAM bytes per launch from an ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of one
@@ -901,9 +901,9 @@ def run_geo(args, wl, world, rank, local_rank):
     stream = torch.cuda.Stream()
     Dd, ud, rd = (torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (D, u_in, r_in))
     out = torch.empty((F, N, E) if node else (F, E, N), device="cuda")
-    cands = [v for v in lc.enumerate_variants(kernel, E, N, F, args.layout, wl["precision"])]
-    if args.variant == "default":
-        cands = [lc.variant_default(kernel, E, N, F, args.layout, wl["precision"])]
+    cands = [lc.variant_default(kernel, E, N, F, args.layout, wl["precision"])]
+    if args.variant != "default":
+        cands += lc.enumerate_variants(kernel, E, N, F, args.layout, wl["precision"])
     best = None
     with torch.cuda.stream(stream):
         for v in cands:
