@@ -127,6 +127,11 @@ lc_status lc_enumerate_variants(const lc_kernel *k, int64_t E, int32_t N, int32_
         if (!any)
             cand = candidates(N, F, layout, LC_PREC_FP32);
     }
+    // the library's default, where the grid above does not hold it
+    lc_variant d;
+    if ((k->k.kind == KIND_CONTRACT || k->k.kind == KIND_GEO) &&
+        lc_variant_default(k, E, N, F, layout, precision, &d) == LC_OK)
+        cand.push_back(d);
     int n = 0;
     for (const lc_variant &v : cand) {
         if (lc_variant_validate(k, E, N, F, &v) != LC_OK)

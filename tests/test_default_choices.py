@@ -91,3 +91,15 @@ def test_short_node_major_rows_keep_the_aligned_plan(kernel, E):
             q = lc.variant_plan(kernel, E, N, F, v)
             for key in ("ops_per_block", "a_buffers", "a_in_tmem", "smem_bytes"):
                 assert q[key] == p[key], (N, F, precision, key)
+
+
+@pytest.mark.parametrize("layout", ["elem", "node"])
+@pytest.mark.parametrize("precision", ["fp32", "fp64", "bf16", "bf16x3"])
+def test_default_is_among_the_candidates(kernel, layout, precision):
+    """The exhaustive autotuner must not miss what a program gets without it."""
+    for N, F in ((4, 1), (4, 6), (20, 2), (35, 3), (50, 1), (66, 3), (84, 4), (120, 3), (165, 3), (200, 1)):
+        for E in (800, 20000, 1 << 21):
+            v = lc.variant_dict(lc.variant_default(kernel, E, N, F, layout, precision))
+            if lc.variant_plan(kernel, E, N, F, lc.Variant(**v))["threads"] >= 64:
+                cands = [lc.variant_dict(c) for c in lc.enumerate_variants(kernel, E, N, F, layout, precision)]
+                assert cands.count(v) == 1, (N, F, E)
