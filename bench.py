@@ -100,23 +100,23 @@ SAXPY_SOURCES = ('frontend.cu', 'lc_internal.h', 'api.cu')
 # full-size launch, keyed by (workload, layout, precision, engine); valid only while the kernel's
 # sources hash to `src`.  `variant` records the descriptor the capture ran.
 NCU_TRAFFIC = {
-    # E = 2^21: 293.77 MB read + 818.33 MB written (the rest of the output still in L2 at the end)
+    # E = 2^21: 293.73 MB read + 818.76 MB written (the rest of the output still in L2 at the end)
     ("fp32_three", "elem", "bf16x3", "tcgen05"): {
-        "bytes": 293_765_120 + 818_326_016, "files": TC_SOURCES, "src": "34f1edfce109485b",
-        "variant": {"tile_e": 128, "elems_per_thread": 64, "split_i": 0, "unroll": 3, "prefetch_smem": 2,
-                    "stages": 1, "store_rows": 128}},
-    # volume derivative, E = 2^21: 369.20 MB read + 818.94 MB written
+        "bytes": 293_730_560 + 818_762_496, "files": TC_SOURCES, "src": "6a63936d16e6717e",
+        "variant": {"tile_e": 128, "elems_per_thread": 1, "split_i": 0, "unroll": 4, "prefetch_smem": 1,
+                    "stages": 3, "store_rows": 128, "a_operand": 1}},
+    # volume derivative, E = 2^21: 369.19 MB read + 818.92 MB written
     ("geo", "elem", "bf16x3", "tcgen05"): {
-        "bytes": 369_195_264 + 818_944_768, "files": GEO_SOURCES, "src": "dd8f4fd0ce0d8bf2",
-        "variant": {"tile_e": 128, "elems_per_thread": 64, "split_i": 0, "unroll": 3, "prefetch_smem": 2,
-                    "stages": 1, "a_operand": 1}},
-    # surface lift, E = 2^21: 830.68 MB read + 267.15 MB written
+        "bytes": 369_189_376 + 818_916_352, "files": GEO_SOURCES, "src": "1ca983392efed0ff",
+        "variant": {"tile_e": 128, "elems_per_thread": 1, "split_i": 0, "unroll": 3, "prefetch_smem": 2,
+                    "stages": 2, "store_rows": 128, "a_operand": 1}},
+    # surface lift, E = 2^21: 830.77 MB read + 261.91 MB written
     ("lift", "elem", "fp32", "simt"): {
-        "bytes": 830_676_736 + 267_149_568, "files": LIFT_SOURCES, "src": "63edc94dc8539bb3",
+        "bytes": 830_770_176 + 261_910_272, "files": LIFT_SOURCES, "src": "75775cc17e068bcd",
         "variant": {"tile_e": 64, "prefetch_smem": 1, "stages": 1, "ctas_per_sm": 3}},
-    # saxpy, n = 2^28: 2147.55 MB read + 1035.85 MB written
+    # saxpy, n = 2^28: 2147.55 MB read + 1036.75 MB written
     ("saxpy", "elem", "fp32", "simt"): {
-        "bytes": 2_147_546_880 + 1_035_845_376, "files": SAXPY_SOURCES, "src": "3af129c596256b81",
+        "bytes": 2_147_546_112 + 1_036_752_896, "files": SAXPY_SOURCES, "src": "30a8cb4a64cccaa9",
         "variant": {"elems_per_thread": 4, "unroll": 4, "ctas_per_sm": 4}},
 }
 

@@ -163,8 +163,8 @@ struct lc_variant {
                                  bandwidth (BF16X3: the products stacked where two accumulators
                                  and the A terms fit tensor memory, one operator up to N = 88,
                                  unless mma_order is 2; else one accumulator region per buffer,
-                                 N up to 128; not for the three-term
-                                 geometric-factor kernel) */
+                                 N up to 128; not for the three-term geometric-factor kernel,
+                                 nor with mma_order 1, which asks for shared memory) */
 };
 
 /*
@@ -348,7 +348,11 @@ lc_status lc_contract_geo(const lc_kernel *k, const lc_variant *v, const void *D
  * memory (u, vmapP and s must then be 16-byte aligned, else every operand is read from
  * global memory, as with prefetch_smem 0); ctas_per_sm (0 = 4) and max_ctas size the
  * persistent grid, which never exceeds the CTAs resident at once; tile_e 64 or 128 elements
- * per tile.  An index out
+ * per tile.  With one buffer, tiles of 64 and staged operands, a kernel that keeps the fluxes
+ * in registers instead serves up to four faces and 64 face nodes where it measured faster (by
+ * E, N, Nf * Nfp and accumulate): one CTA per SM with tiles of up to eight warps' elements and
+ * a window of 64 to 256 rows on either side; max_ctas bounds it too, ctas_per_sm is unused.
+ * An index out
  * of range is not followed: its flux becomes NaN and lc_device_error reports LC_ERR_INDEX.
  * Errors: LC_ERR_INVALID_ARGUMENT, LC_ERR_INVALID_VARIANT, LC_ERR_MISALIGNED (4-byte),
  * LC_ERR_NO_DEVICE, LC_ERR_UNSUPPORTED (not a kernel of this form), LC_ERR_CUDA.
@@ -455,8 +459,9 @@ lc_status lc_grouped_plan_create(const lc_kernel *k, const lc_variant *v, const 
 /* Enqueue the planned launch (graph replay when captured) on `stream`. */
 lc_status lc_grouped_run(lc_grouped_plan *plan, void *stream);
 
-/* Grid size (both launches) and number of (group, tile-range) segments of a plan (a
- * tensor-core CTA counts as one segment). */
+/* Grid size (all launches of the plan together) and number of (group, tile-range) segments (a
+ * tensor-core CTA, of the grouped launch or of a group's own, counts as one segment; K-split
+ * launches add none). */
 lc_status lc_grouped_plan_info(const lc_grouped_plan *plan, int32_t *grid, int32_t *segments);
 
 /*
@@ -522,7 +527,7 @@ lc_status lc_autotune(const lc_kernel *k, int64_t E, int32_t N, int32_t F, int32
 
 /*
  * MLP cost model: inputs x[din] (1 <= din <= 32), three hidden ReLU layers of width
- * 64, one linear output (the predicted log run time).  Parameters are one float
+ * 64, one linear output (the score the network was trained on).  Parameters are one float
  * vector, in this order: W1[64][din], b1[64], W2[64][64], b2[64], W3[64][64], b3[64],
  * w4[64], b4[1]; all pointers below are device pointers, arrays row-major.
  */
@@ -572,10 +577,12 @@ lc_status lc_pick_workspace_size(size_t *bytes);
 
 /*
  * Pick a descriptor with a trained cost model: enumerate the candidates
- * (lc_enumerate_variants), build their features (lc_variant_features), predict their log
- * run time with lc_mlp_forward on `stream` (din = LC_FEATURES), and return the candidate
- * with the smallest prediction (the first one on ties) in *picked, its prediction in
- * *predicted (may be NULL).  Synchronises `stream`.
+ * (lc_enumerate_variants), build their features (lc_variant_features), score them
+ * with lc_mlp_forward on `stream` (din = LC_FEATURES), and return the candidate with the
+ * smallest score (the first one on ties) in *picked, its score in *predicted (may be NULL).
+ * What the score means is the training target's affair (a log run time, a slowdown against
+ * the problem's best candidate): it only has to grow with the run time among the candidates
+ * of one problem.  Synchronises `stream`.
  *   params_dev     the network's parameters (lc_mlp_param_count(LC_FEATURES) floats)
  *   workspace_dev  lc_pick_workspace_size bytes, 16-byte aligned (features, predictions)
  * Errors: LC_ERR_INVALID_ARGUMENT, LC_ERR_BUFFER_TOO_SMALL, LC_ERR_MISALIGNED,
@@ -588,7 +595,7 @@ lc_status lc_pick_variant(const lc_kernel *k, int64_t E, int32_t N, int32_t F, i
 /*
  * lc_pick_variant with an ensemble of n_models networks of the same shape, trained apart
  * (different initialisations and minibatch orders): each candidate's prediction is the mean
- * of the models' predicted log run times (models taken in order), and the candidate with
+ * of the models' scores (models taken in order), and the candidate with
  * the smallest mean is returned (*predicted = that mean).  Averaging removes much of one
  * network's variance between trainings (held-out regret of single networks differs by
  * several points from seed to seed).  lc_pick_variant is the case n_models = 1.

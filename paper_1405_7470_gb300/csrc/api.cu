@@ -1227,8 +1227,8 @@ static lc_status resolve(const Kernel &K, long long E, int N, int F, const lc_va
         // small N (few, large stores), else 32-row pieces of one operator at a time (the
         // stores stream, and the staging slots stay small)
         t.store_quarters = geo ? 4 : (v->store_rows ? v->store_rows / 32 : (N <= 48 ? 4 : 1));
-        // a_tm: A terms in tensor memory (one accumulator region each: BF16, or BF16X3 with the
-        // hi*hi products last), else in shared memory
+        // a_tm: A terms in tensor memory (BF16; BF16X3 stacked where the columns allow it, else in one
+        // accumulator region with the hi*hi products last), else in shared memory
         auto plan = [&](int G, TcArgs &q, bool a_tm) -> bool {
             q.G = G;
             // operator padding: 16 columns (16-column epilogue chunks), or 8 where that lets
@@ -1306,9 +1306,9 @@ static lc_status resolve(const Kernel &K, long long E, int N, int F, const lc_va
         const int g_hi = v->split_i ? v->split_i : F, g_lo = geo ? F : (v->split_i ? v->split_i : 1);
         // the most operators per CTA first; for each, the planner's A placement first: tensor
         // memory for BF16 (it frees shared memory for stages and slots), shared memory for
-        // BF16X3 (the stacked order needs both accumulators' columns, and a long chain of MMAs
-        // reading A from tensor memory measured slower beside the epilogue's loads); BF16X3
-        // takes tensor-memory A where no shared-memory plan fits (N above about 100)
+        // BF16X3 (more operators of a block fit stacked there: 2 CBp <= 256, beside tensor-memory
+        // A terms one operator up to N = 88), which takes tensor-memory A where no shared-memory
+        // plan fits (N above about 100) or where the descriptor asks for it
         const bool tm_first = v->a_operand == 2 || (v->a_operand == 0 && NT == 1);
         // (node-major rows that are not 16-byte aligned need stage rows of 132 values; where that
         // does not fit, or no tile has a 132nd value, the tiles are read from global memory)
@@ -2567,7 +2567,7 @@ static lc_status grouped_plan_host(const Kernel &K, const lc_variant *v, const l
             const double pad = (double)(r.g.nchunks * (long long)r.g.CW) / ((double)G.F * G.N) - 1.0;
             const bool nodel = v->layout == LC_LAYOUT_NODE_MAJOR;
             // node-major: the tile the autotuner measured fastest for the plain SIMT kernel at
-            // this N (lc_variant_default) comes first (grouped, full-size uneven batching: 7.9
+            // this N came first (grouped, full-size uneven batching: 7.9
             // against 8.5 ms; element-major kept the weighted sum: 6.2 against 6.6 ms); the
             // weighted sum orders the rest
             const int pref = nodel ? (G.N <= 40 ? 128 : G.N <= 72 ? 64 : 32) : 0;

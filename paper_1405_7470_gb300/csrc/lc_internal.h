@@ -243,13 +243,13 @@ int current_cc(int *major, int *minor);
 unsigned int *error_word();
 lc_status cuda_fail(cudaError_t e);
 size_t smem_optin_limit();
-
-// SIMT launchers (one per element type / layout translation unit).
 // Let kernel `fn` be launched with any plan's dynamic shared memory.  Always the device's limit, not one
 // plan's size: the attribute belongs to the function, so a smaller plan on the same instance (another
 // thread's, or any call between a grouped plan's creation and its run) would make the larger plan's
 // launch fail.  (No kernel that uses it has static shared memory, which counts against the limit.)
 cudaError_t allow_smem(const void *fn);
+
+// SIMT launchers (one per element type / layout translation unit).
 lc_status simt_launch_f32_elem(const SimtArgs &a, const SimtGeom &g, int unroll, int prefetch,
                                cudaStream_t s);
 lc_status simt_launch_f32_node(const SimtArgs &a, const SimtGeom &g, int unroll, int prefetch,

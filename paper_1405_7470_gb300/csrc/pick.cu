@@ -132,7 +132,7 @@ lc_status lc_pick_variant_ensemble(const lc_kernel *k, int64_t E, int32_t N, int
     cudaError_t e = cudaMemcpyAsync(Xd, X.data(), sizeof(float) * X.size(), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess)
         return lc::cuda_fail(e);
-    // the models' predicted log times, averaged in model order
+    // the models' predictions, averaged in model order
     for (int q = 0; q < n_models; ++q) {
         st = lc_mlp_forward(params_dev + (size_t)q * P, Xd, n, LC_FEATURES, yd, stream);
         if (st != LC_OK)

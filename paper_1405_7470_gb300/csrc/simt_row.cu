@@ -26,8 +26,9 @@
 // a chunk is a unit of its own.
 // Measured, F = 3, E = 2^21, before (simt.cuh) -> after: N = 35 element-major 494 -> 351 us (HBM floor
 // 175, FMA floor 191), node-major 486 -> 356; N = 20 280 -> 121 and 228 -> 142 (HBM floor 100).  At
-// N = 35 the FMA pipes are 53 % busy: a warp's own dependent issue (two warps an SMSP, all the
-// registers allow) and the wait for its next rows are what is left.
+// N = 35 the FMA pipes are 53 % busy, the load/store wavefronts 33 %, and an instruction issues in
+// 39 % of the cycles: the largest stall is the fixed latency of a warp's own instructions (two
+// warps an SMSP, all the registers allow), then the wait for its next rows.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -333,9 +333,9 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
     const int N = a.N, G = a.G, CBp = a.CBp, CBs = a.CBs, KB = a.KB, nkb = a.nkb;
     // The A terms in tensor memory are compiled into the BF16 instances and into separate
     // three-term instances (ATM): in the three-term instances for shared-memory A, the
-    // warp-uniform conversion loops the tensor-memory stores need measured slower, and with
-    // three terms the A reads from tensor memory are slower beside the epilogue's loads, so
-    // those plans take them only where the shared-memory plan does not fit (large N).
+    // warp-uniform conversion loops the tensor-memory stores need measured slower.  Three terms
+    // take them where shared memory's bandwidth is the bound (N = 65 to 88), where they keep
+    // every operator in one block, and where no shared-memory plan fits (N above about 100).
     constexpr bool kATmem = ATM;
     const int Np = a.Np;  // accumulator columns per operator (N rounded up to 16)
     // K columns the MMAs read: N rounded up to the 16 of one instruction.  A K-block
@@ -775,7 +775,7 @@ __device__ __forceinline__ void tc_body(const TcArgs &a, const int blk, const lo
                 if (lane == 0)
                     mbar_arrive(&a_full[ab * kTcMaxKB + kb]);
             };
-            // chunks c8, c8 + Hc, ... below c8_hi, two in flight (uniform across the warp: tcgen05.st
+            // chunks c8, c8 + Hc, ... below c8_hi, one at a time (uniform across the warp: tcgen05.st
             // is warp-collective)
             auto convert = [&](auto staged, int c8, int c8_hi) {
                 for (; c8 < c8_hi; c8 += Hc) {

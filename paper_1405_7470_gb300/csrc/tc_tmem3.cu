@@ -1,6 +1,5 @@
-// Tensor-core contraction, three-term split (BF16X3) with the A terms in tensor memory: the
-// plans for large N whose shared-memory plan does not fit (both layouts, both epilogue chunk
-// widths).  The kernel template is in tc.cuh.
+// Tensor-core contraction, three-term split (BF16X3) with the A terms in tensor memory (both
+// layouts, both epilogue chunk widths).  The kernel template is in tc.cuh.
 #include "tc.cuh"
 
 namespace lc {

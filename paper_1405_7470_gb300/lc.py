@@ -452,7 +452,7 @@ def variant_features(kernel: Kernel, E: int, N: int, F: int, layout, precision, 
 
 
 def pick_variant(kernel: Kernel, E: int, N: int, F: int, layout, precision, params, workspace=None, stream=None):
-    """(descriptor, predicted log ms) picked by the trained network `params` (lc_pick_variant),
+    """(descriptor, its predicted score, lower is better) picked by the trained network `params` (lc_pick_variant),
     or by an ensemble when `params` is 2-D, one network's parameters per row
     (lc_pick_variant_ensemble)."""
     import torch

@@ -141,7 +141,8 @@ def dataset(recs):
     """Features and targets: the square root of each candidate's log slowdown against its shape's
     best, cut at 1.  The pick only compares candidates of one shape, so the network need not learn
     how long a shape takes, nor how bad a candidate is beyond e times the best; the root spreads
-    out the good ones.  (Held-out regret, geo-mean: 2 to 3 % against 2 to 7 % with the log time.)"""
+    out the good ones.  (Held-out regret, geo-mean, 100 shapes that took no part in the choice of
+    the target: 2.7 and 4.1 % in two runs; 4.8 % with the log time on earlier kernels.)"""
     X, y = [], []
     for r in recs:
         best = max(min(ms for ms, _ in r["cands"]), 1e-4)
