@@ -1311,8 +1311,11 @@ static lc_status resolve(const Kernel &K, long long E, int N, int F, const lc_va
         // plan fits (N above about 100) or where the descriptor asks for it
         const bool tm_first = v->a_operand == 2 || (v->a_operand == 0 && NT == 1);
         // (node-major rows that are not 16-byte aligned need stage rows of 132 values; where that
-        // does not fit, or no tile has a 132nd value, the tiles are read from global memory)
-        for (int shifted = node && E % 4 != 0 && E >= 132 ? 1 : 0; shifted >= 0 && !found; --shifted)
+        // does not fit, no tile has a 132nd value, or one stage holds few short rows, the tiles are
+        // read from global memory: one stage, BF16, N = 4, F = 1, E = 6250001 399 us against 447,
+        // N = 16, F = 3 85 against 92, N = 20, F = 2 113 against 105; with two stages copies always win)
+        const bool copies = v->stages > 1 || N > 16;
+        for (int shifted = node && E % 4 != 0 && E >= 132 && copies ? 1 : 0; shifted >= 0 && !found; --shifted)
         for (int g = g_hi; g >= g_lo && !found; --g)
             for (int pass = 0; pass < 2 && !found; ++pass) {
                 const bool a_tm = tm_first ? pass == 0 : pass == 1;

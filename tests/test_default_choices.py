@@ -103,3 +103,14 @@ def test_default_is_among_the_candidates(kernel, layout, precision):
             if lc.variant_plan(kernel, E, N, F, lc.Variant(**v))["threads"] >= 64:
                 cands = [lc.variant_dict(c) for c in lc.enumerate_variants(kernel, E, N, F, layout, precision)]
                 assert cands.count(v) == 1, (N, F, E)
+
+
+@pytest.mark.parametrize("N,stages,copies", [(4, 1, False), (16, 1, False), (17, 1, True), (35, 1, True), (16, 2, True),
+                                             (16, 3, True)])
+def test_one_stage_of_short_unaligned_rows_is_read_directly(kernel, N, stages, copies):
+    """Node-major rows off the 16-byte boundary: bulk copies take stage rows of 132 values, 16 bytes more (before
+    the parts are aligned)."""
+    v = lc.Variant(engine="tcgen05", layout="node", precision="bf16x3", tile_e=128, elems_per_thread=64, split_i=0,
+                   unroll=3, prefetch_smem=1, stages=stages)
+    aligned, odd = (lc.variant_plan(kernel, E, N, 2, v)["smem_bytes"] for E in (4000, 4001))
+    assert (odd > aligned) if copies else (odd == aligned)
