@@ -100,23 +100,23 @@ SAXPY_SOURCES = ('frontend.cu', 'lc_internal.h', 'api.cu')
 # full-size launch, keyed by (workload, layout, precision, engine); valid only while the kernel's
 # sources hash to `src`.  `variant` records the descriptor the capture ran.
 NCU_TRAFFIC = {
-    # E = 2^21: 293.73 MB read + 818.76 MB written (the rest of the output still in L2 at the end)
+    # E = 2^21: 293.69 MB read + 818.54 MB written (the rest of the output still in L2 at the end)
     ("fp32_three", "elem", "bf16x3", "tcgen05"): {
-        "bytes": 293_730_560 + 818_762_496, "files": TC_SOURCES, "src": "6a63936d16e6717e",
+        "bytes": 293_692_672 + 818_542_336, "files": TC_SOURCES, "src": "f63acf1de78d6cb9",
         "variant": {"tile_e": 128, "elems_per_thread": 1, "split_i": 0, "unroll": 4, "prefetch_smem": 1,
                     "stages": 3, "store_rows": 128, "a_operand": 1}},
-    # volume derivative, E = 2^21: 369.19 MB read + 818.92 MB written
+    # volume derivative, E = 2^21: 369.24 MB read + 818.89 MB written
     ("geo", "elem", "bf16x3", "tcgen05"): {
-        "bytes": 369_189_376 + 818_916_352, "files": GEO_SOURCES, "src": "1ca983392efed0ff",
+        "bytes": 369_238_272 + 818_887_168, "files": GEO_SOURCES, "src": "df9bc0e5e853f87a",
         "variant": {"tile_e": 128, "elems_per_thread": 1, "split_i": 0, "unroll": 3, "prefetch_smem": 2,
                     "stages": 2, "store_rows": 128, "a_operand": 1}},
-    # surface lift, E = 2^21: 830.77 MB read + 261.91 MB written
+    # surface lift, E = 2^21: 830.61 MB read + 262.03 MB written
     ("lift", "elem", "fp32", "simt"): {
-        "bytes": 830_770_176 + 261_910_272, "files": LIFT_SOURCES, "src": "75775cc17e068bcd",
+        "bytes": 830_606_848 + 262_025_728, "files": LIFT_SOURCES, "src": "c16e2ebe1c7cb966",
         "variant": {"tile_e": 64, "prefetch_smem": 1, "stages": 1, "ctas_per_sm": 3}},
-    # saxpy, n = 2^28: 2147.55 MB read + 1036.75 MB written
+    # saxpy, n = 2^28: 2147.52 MB read + 1036.88 MB written
     ("saxpy", "elem", "fp32", "simt"): {
-        "bytes": 2_147_546_112 + 1_036_752_896, "files": SAXPY_SOURCES, "src": "30a8cb4a64cccaa9",
+        "bytes": 2_147_516_160 + 1_036_876_288, "files": SAXPY_SOURCES, "src": "d85adf9a2588d8cf",
         "variant": {"elems_per_thread": 4, "unroll": 4, "ctas_per_sm": 4}},
 }
 
